@@ -75,7 +75,8 @@ int poly_diag_fields(void* plan, const void* delta_x, void* fields_host, void* s
  *   Each other pointer may be NULL (not written) or a caller-owned host buffer:
  *   bins      int32 [nbins][order], 1-based shells;
  *   tiles     int32 [ntiles][8]: row_off, nrow, col_off, ncol, field_off, nfield,
- *             region_mask (bit (r / 32) * 4 + c / 16), padding;
+ *             region_mask (bit (r / 32) * 4 + c / 16), padding: one tile per task of
+ *             the FP64 contraction, its fields the runs of shells of the task's legs;
  *   field_ids int32, 0-based field slots, tile t's at field_off .. + nfield;
  *   rowf/colf int16 [][4]: up to three tile-local field indices (-1: none),
  *             row r of tile t at rowf[row_off + r], column c at colf[col_off + c];

@@ -1,14 +1,33 @@
 // CUDA-core contraction over grid cells (Eq. estimator, discrete form of App. A):
 //   S_b = sum_x prod_t D_{b_t}(x)
-// recast per tile as a GEMM  C[r][c] = sum_x A_r(x) B_c(x), where a row A_r is a
-// product of one to three shell fields (e.g. D_{k1} D_{k2}) and a column B_c the
-// product of the remaining ones (D_{k3}, D_{k3} D_{k4}, or three for n = 5, 6).  Cells are split
-// across blocks (split-K); every block writes its FP64 partial tile and a
-// fixed-order reduction gathers the bins.
 //
-// FP32 instantiation: products and per-chunk accumulation in FP32, flushed to
-// FP64 every kFlushChunks chunks.  FP64 instantiation: FP64 throughout (the
-// plain method, and the exact polygon counts over the symmetry wedge).
+// A task is a block of bins: one run of consecutive shells per leg (e.g. 4 x 4 x 4
+// for FP32 bispectra), rows the products of the first legs and columns the
+// products of the rest.  One warp takes a task and its lanes the cells: each lane
+// loads one value (FP32: of two neighbouring cells) per field of the task's runs,
+// forms the row and column products in registers and adds every row times every
+// column to its own accumulators, kept in registers over all of the warp's cells.
+// FP32 arithmetic runs in packed pairs, one cell in each half, so that no operand
+// has to be duplicated.
+//
+// What bounds it: FMA issue.  The block over three legs needs 24 shared-memory
+// wavefronts (4 + 4 + 4 fields, conflict-free rows of the cell-tiled layout) for
+// 64 + 16 packed multiply-adds and products, 60 % of the shared memory's rate at
+// the FP32 FMA peak.  (A 64 x 64 tile of products staged in shared memory, 4 x 4
+// per lane and two 16-byte loads per 16 FMAs, is bound by those loads at 50 % of the
+// peak before the products and the idle parts of the tile: 121 ms at 256^3 / 64
+// shells against 36 ms here, 38 TFLOP/s of a measured 56 to 66 TFLOP/s of packed
+// FMAs over such register blocks; FP64 at 64^3 / 16 shells 1.05 against 0.45 ms.)
+// The blocks follow the bins closely: 508 tasks x 64 = 1.33 products per bin at
+// 24,432 triangles.
+//
+// Fields of one block's tasks arrive by 16-byte asynchronous copies of every thread
+// (stages of a few chunks) and serve its 12 warps; one bulk copy per run of fields
+// and chunk, about a KB each, took 58 ms.  FP32 lane sums cover 256 steps; then they
+// are summed over the warp and added to FP64 sums.  FP64 throughout for the plain
+// method and the exact polygon counts over the symmetry wedge (cell weights on the
+// rows).
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -16,155 +35,234 @@
 
 namespace ps {
 
-constexpr int kCcThreads = 256;
-constexpr int kFlushChunks = 32;  // 32 chunks x 32 cells = 1024 cells per FP32 partial sum
+constexpr int kCcWarps = kCcTasksPerGroup;                          // task warps per block
+constexpr int kCcThreads = kCcWarps * 32;
+constexpr int kCcFlush = 256;  // steps per FP32 partial sum
 
-PS_DEV void load4(const float* p, float* v) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+PS_DEV void cc_copy16(uint32_t dst_smem, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
 }
-PS_DEV void load4(const double* p, double* v) {
-    const double2 q0 = reinterpret_cast<const double2*>(p)[0], q1 = reinterpret_cast<const double2*>(p)[1];
-    v[0] = q0.x, v[1] = q0.y, v[2] = q1.x, v[3] = q1.y;
+PS_DEV void cc_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+PS_DEV void cc_wait() {  // all but this thread's last LEFT groups of copies have landed
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
 }
 
-// NF: factors per row or column at most (2 for n <= 4, 3 for n = 5, 6); the third is never read for NF = 2.
-template <typename T, bool WEIGHTED, bool ABS, int NF>
-__global__ void __launch_bounds__(kCcThreads) contract_cc_kernel(
-    const T* __restrict__ fields, size_t fstride, int tile_ns, int64_t ncell, const T* __restrict__ weight,
-    const PsTile* __restrict__ tiles, int ntiles, const int* __restrict__ field_ids, const short4* __restrict__ rowf,
-    const short4* __restrict__ colf, int64_t chunks_per_split, double* __restrict__ partial) {
-    constexpr int CH = sizeof(T) == 8 ? 16 : 32, TM = kCcTM, TN = kCcTN;
-    __shared__ T s_d[kCcMaxFields][CH + 1];
-    __shared__ __align__(16) T s_a[CH][TM];
-    __shared__ __align__(16) T s_b[CH][TN];
-    using FT = typename std::conditional<NF == 3, short4, short2>::type;  // factor record in shared memory
-    __shared__ FT s_rf[TM], s_cf[TN];
-    __shared__ int s_fid[kCcMaxFields];
+// What a lane holds of one field in one step: two cells (FP32) or one (FP64).
+template <typename T>
+struct CcLane;
+template <>
+struct CcLane<float> {
+    using V = unsigned long long;  // two floats; as one 64-bit value they stay in an aligned register pair without moves
+    static constexpr int kChunks = 2;  // 32-cell chunks of a step: lanes 0-15 take the first, 16-31 the second
+    static PS_DEV uint32_t offset(int lane, int chunk_bytes) { return (uint32_t)((lane >> 4) * chunk_bytes + (lane & 15) * 8); }
+    static PS_DEV V zero() { return 0ull; }
+    static PS_DEV V load(uint32_t a) {
+        V v;
+        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(a));
+        return v;
+    }
+    static PS_DEV V mul(V a, V b) {
+        V r;
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+        return r;
+    }
+    static PS_DEV V mad(V a, V b, V c) {
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+        return c;
+    }
+    static PS_DEV V abs(V a) { return a & 0x7fffffff7fffffffull; }
+    static PS_DEV float sum(V a) { return __uint_as_float((uint32_t)a) + __uint_as_float((uint32_t)(a >> 32)); }
+};
+template <>
+struct CcLane<double> {
+    using V = double;
+    static constexpr int kChunks = 1;
+    static PS_DEV uint32_t offset(int lane, int) { return (uint32_t)(lane * 8); }
+    static PS_DEV V zero() { return 0.0; }
+    static PS_DEV V load(uint32_t a) {
+        V v;
+        asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
+        return v;
+    }
+    static PS_DEV V mul(V a, V b) { return a * b; }
+    static PS_DEV V mad(V a, V b, V c) { return fma(a, b, c); }
+    static PS_DEV V abs(V a) { return fabs(a); }
+    static PS_DEV double sum(V a) { return a; }
+};
 
-    const PsTile tile = tiles[blockIdx.x];
-    const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
-    // warp w owns the 32x16 region (rows 32*(w/4).., cols 16*(w%4)..), lane -> 4x4 sub-block
-    const int r0 = 32 * (warp >> 2) + 4 * (lane >> 2);
-    const int c0 = 16 * (warp & 3) + 4 * (lane & 3);
-    const bool active = (tile.region_mask >> warp) & 1u;
+// The products of one value per leg of legs [L0, L1), the first leg's index slowest; leg l's values at d[S::at(l)].
+template <typename T, class S, int L0, int L1>
+PS_DEV void cc_products(const typename CcLane<T>::V* d, typename CcLane<T>::V* o) {
+    constexpr int D = S::dim(L1 - 1), n = S::span(L0, L1 - 1), at = S::at(L1 - 1);
+    if constexpr (L1 - L0 == 1) {
+#pragma unroll
+        for (int i = 0; i < D; i++) o[i] = d[at + i];
+    } else {
+        typename CcLane<T>::V h[n];
+        cc_products<T, S, L0, L1 - 1>(d, h);
+#pragma unroll
+        for (int a = 0; a < n; a++)
+#pragma unroll
+            for (int i = 0; i < D; i++) o[a * D + i] = CcLane<T>::mul(h[a], d[at + i]);
+    }
+}
 
-    auto narrow = [](short4 f) {
-        if constexpr (NF == 3) return f;
-        else return make_short2(f.x, f.y);
-    };
-    const short4 none = make_short4(-1, -1, -1, -1);
-    for (int i = tid; i < TM; i += kCcThreads) s_rf[i] = narrow(i < tile.nrow ? rowf[tile.row_off + i] : none);
-    for (int i = tid; i < TN; i += kCcThreads) s_cf[i] = narrow(i < tile.ncol ? colf[tile.col_off + i] : none);
-    for (int i = tid; i < tile.nfield; i += kCcThreads) s_fid[i] = field_ids[tile.field_off + i];
-
-    T acc[4][4];
-    double acc64[4][4];
+// Sum of V values over the warp's 32 lanes by halving: after the exchange at lane distance d a
+// lane keeps the half of the values that its bit d selects.  V = 64: lane l ends with values
+// 2 l' and 2 l' + 1, l' = the bits of l (16 first) as the high bits of the value index.
+template <typename T, int V>
+PS_DEV void cc_warp_sum(T* v, int lane) {
+    int n = V;
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int d = 16; d > 0; d >>= 1) {
+        const bool up = lane & d;
+        if (n > 1) {
+            n >>= 1;
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            acc[i][j] = 0;
-            acc64[i][j] = 0.0;
-        }
-
-    const int64_t nchunks = (ncell + CH - 1) / CH;
-    const int64_t cbeg = (int64_t)blockIdx.y * chunks_per_split;
-    const int64_t cend = min(nchunks, cbeg + chunks_per_split);
-    __syncthreads();
-    // register prefetch of the next chunk's field values (each thread owns a fixed set of (f, x))
-    constexpr int PF = kCcMaxFields * CH / kCcThreads;
-    const int nload = tile.nfield * CH;
-    T pf[PF];
-    auto fetch = [&](int64_t ch) {
-#pragma unroll
-        for (int k = 0; k < PF; k++) {
-            const int e = tid + k * kCcThreads;
-            if (e < nload) {
-                const int f = e / CH, x = e - (e / CH) * CH;
-                const int64_t cell = ch * CH + x;
-                const size_t a = tile_ns > 0 ? (size_t)(cell >> 5) * tile_ns * 32 + (size_t)s_fid[f] * 32 + (cell & 31)
-                                             : (size_t)s_fid[f] * fstride + cell;
-                pf[k] = (ch < cend && cell < ncell) ? fields[a] : (T)0;
-            }
-        }
-    };
-    // the row and column this thread forms products for are the same in every chunk
-    static_assert(kCcThreads % TM == 0 && kCcThreads % TN == 0, "rows and columns per thread must not vary");
-    const int r = tid % TM, c = tid % TN;
-    const FT frow = s_rf[r], fcol = s_cf[c];
-    if (cbeg < cend) fetch(cbeg);
-    int since_flush = 0;
-    for (int64_t ch = cbeg; ch < cend; ch++) {
-        const int64_t base = ch * CH;
-        // 1. this chunk's field values into shared memory, then prefetch the next chunk
-#pragma unroll
-        for (int k = 0; k < PF; k++) {
-            const int e = tid + k * kCcThreads;
-            if (e < nload) s_d[e / CH][e - (e / CH) * CH] = pf[k];
-        }
-        __syncthreads();
-        fetch(ch + 1);
-        // 2. row and column products
-        for (int x = tid / TM; x < CH; x += kCcThreads / TM) {  // this thread's row r, every cell x it owns
-            const FT f = frow;
-            T v = 0;
-            if (f.x >= 0) {
-                v = s_d[f.x][x];
-                if (f.y >= 0) v *= s_d[f.y][x];
-                if constexpr (NF == 3)
-                    if (f.z >= 0) v *= s_d[f.z][x];
-                if (WEIGHTED) {
-                    const int64_t cell = base + x;
-                    v *= cell < ncell ? weight[cell] : (T)0;
+            for (int i = 0; i < V / 2; i++)
+                if (i < n) {
+                    const T keep = up ? v[i + n] : v[i], give = up ? v[i] : v[i + n];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, give, d);
                 }
-                if (ABS) v = v < 0 ? -v : v;
-            }
-            s_a[x][r] = v;
-        }
-        for (int x = tid / TN; x < CH; x += kCcThreads / TN) {
-            const FT f = fcol;
-            T v = 0;
-            if (f.x >= 0) {
-                v = s_d[f.x][x];
-                if (f.y >= 0) v *= s_d[f.y][x];
-                if constexpr (NF == 3)
-                    if (f.z >= 0) v *= s_d[f.z][x];
-                if (ABS) v = v < 0 ? -v : v;
-            }
-            s_b[x][c] = v;
-        }
-        __syncthreads();
-        // 3. 4x4 outer products per lane over the chunk (16-byte vector loads)
-        if (active) {
-#pragma unroll 8
-            for (int x = 0; x < CH; x++) {
-                T a[4], b[4];
-                load4(&s_a[x][r0], a);
-                load4(&s_b[x][c0], b);
-#pragma unroll
-                for (int i = 0; i < 4; i++)
-#pragma unroll
-                    for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-            }
-        }
-        if (sizeof(T) == 4 && ++since_flush == kFlushChunks) {
-            since_flush = 0;
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    acc64[i][j] += (double)acc[i][j];
-                    acc[i][j] = 0;
-                }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
         }
     }
-    double* out = partial + ((size_t)blockIdx.y * ntiles + blockIdx.x) * (TM * TN);
+}
+
+template <typename T, int ORDER, bool WEIGHTED, bool ABS>
+__global__ void __launch_bounds__(kCcThreads, 1)
+    contract_cc_kernel(const T* __restrict__ fields, int nf, int64_t nchunk, const T* __restrict__ weight,
+                       const CcGroup* __restrict__ groups, int ngroups, const CcTask* __restrict__ tasks, int64_t ntask,
+                       int nsplit, int wpt, int stage_chunks, int stage_bytes, double* __restrict__ partial) {
+    using S = CcShape<ORDER, sizeof(T) == 8>;
+    using Ln = CcLane<T>;
+    using LV = typename Ln::V;
+    constexpr int RA = S::ra, V = S::rows * S::cols;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gi = blockIdx.x % ngroups, split = blockIdx.x / ngroups;
+    const CcGroup* grp = groups + gi;
+    const int used = grp->used, task_off = grp->task_off, tpg = grp->ntask;
+    // the block's chunks (whole steps), in stages
+    const int64_t nstep = nchunk / Ln::kChunks;
+    const int64_t c0 = nstep * split / nsplit * Ln::kChunks, c1 = nstep * (split + 1) / nsplit * Ln::kChunks;
+    const int nst = (int)((c1 - c0 + stage_chunks - 1) / stage_chunks);
+    const int row_bytes = 32 * (int)sizeof(T);
+    const int chunk_bytes = used * row_bytes;
+
+    // copies of stage `it`: eight threads per field row, 32 rows at a time, chunk by chunk
+    const uint32_t smem = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    constexpr int kPieces = 32 * sizeof(T) / 16 / 8;  // 16-byte pieces of a row per thread
+    auto copy_stage = [&](int it) {
+        const int64_t c = c0 + (int64_t)it * stage_chunks;
+        const int cnt = (int)(c1 - c < stage_chunks ? c1 - c : stage_chunks);
+        for (int u = threadIdx.x >> 3; u < used; u += kCcThreads / 8) {
+            uint32_t dst = smem + (uint32_t)((it % kCcStages) * stage_bytes + u * row_bytes + (threadIdx.x & 7) * 16);
+            const char* src = (const char*)(fields + ((size_t)c * nf + grp->slot[u]) * 32) + (threadIdx.x & 7) * 16;
+            for (int k = 0; k < cnt; k++) {
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+                for (int i = 0; i < kPieces; i++) cc_copy16(dst + i * 128, src + i * 128);
+                dst += chunk_bytes;
+                src += (size_t)nf * row_bytes;
+            }
+        }
+    };
+    for (int it = 0; it < kCcStages - 1; it++) {
+        if (it < nst) copy_stage(it);
+        cc_commit();
+    }
+    // ---------------------------------------------------------------- tasks
+    const int ti = warp % tpg, phase = warp / tpg;  // warps beyond tpg * wpt only copy
+    const bool active = phase < wpt;
+    CcTask task;
 #pragma unroll
-        for (int j = 0; j < 4; j++) out[(r0 + i) * TN + c0 + j] = acc64[i][j] + (double)acc[i][j];
+    for (int l = 0; l < ORDER; l++) {
+        task.row[l] = tasks[task_off + ti].row[l] * (int)sizeof(T);
+    }
+    LV acc[S::rows][S::cols];
+    double acc64[(V + 31) / 32];
+#pragma unroll
+    for (int i = 0; i < S::rows; i++)
+#pragma unroll
+        for (int j = 0; j < S::cols; j++) acc[i][j] = Ln::zero();
+#pragma unroll
+    for (int i = 0; i < (V + 31) / 32; i++) acc64[i] = 0.0;
+
+    auto flush = [&]() {
+        T v[V];
+#pragma unroll
+        for (int i = 0; i < S::rows; i++)
+#pragma unroll
+            for (int j = 0; j < S::cols; j++) {
+                v[i * S::cols + j] = Ln::sum(acc[i][j]);
+                acc[i][j] = Ln::zero();
+            }
+        cc_warp_sum<T, V>(v, lane);
+#pragma unroll
+        for (int i = 0; i < (V + 31) / 32; i++) acc64[i] += (double)v[i];
+    };
+
+    const uint32_t p0 = smem + Ln::offset(lane, chunk_bytes);
+    const int step_bytes = Ln::kChunks * chunk_bytes;
+    int next = phase, since = 0;  // this warp's next step (of the block's range), at least the steps since the last flush
+    for (int it = 0; it < nst; it++) {
+        cc_wait<kCcStages - 2>();  // stage it has landed
+        __syncthreads();           // for every thread, and stage it - 1 has been read by every warp
+        if (it + kCcStages - 1 < nst) copy_stage(it + kCcStages - 1);
+        cc_commit();
+        const int s = it % kCcStages;
+        const int spst = stage_chunks / Ln::kChunks, b0 = it * spst;  // steps of a stage, its first step
+        const int left = (int)((c1 - c0) / Ln::kChunks) - b0, cnt = left < spst ? left : spst;
+        if (active) {
+            int k = next - b0;
+            uint32_t p = p0 + (uint32_t)(s * stage_bytes + k * step_bytes);
+            for (; k < cnt; k += wpt, p += (uint32_t)(wpt * step_bytes)) {
+                LV d[S::nval], rows[S::rows], col[S::cols];
+#pragma unroll
+                for (int l = 0; l < ORDER; l++)
+#pragma unroll
+                    for (int i = 0; i < S::dim(l); i++)
+                        d[S::at(l) + i] = Ln::load(p + task.row[l] + 32 * i * (uint32_t)sizeof(T));
+                cc_products<T, S, 0, RA>(d, rows);
+                cc_products<T, S, RA, ORDER>(d, col);
+                if constexpr (WEIGHTED) {
+                    const T w = weight[(c0 + b0 + k) * 32 + lane];
+#pragma unroll
+                    for (int i = 0; i < S::rows; i++) rows[i] = Ln::mul(rows[i], w);
+                }
+                if constexpr (ABS) {
+#pragma unroll
+                    for (int i = 0; i < S::rows; i++) rows[i] = Ln::abs(rows[i]);
+#pragma unroll
+                    for (int j = 0; j < S::cols; j++) col[j] = Ln::abs(col[j]);
+                }
+#pragma unroll
+                for (int i = 0; i < S::rows; i++)
+#pragma unroll
+                    for (int j = 0; j < S::cols; j++) acc[i][j] = Ln::mad(rows[i], col[j], acc[i][j]);
+            }
+            since += cnt;
+            next = b0 + k;
+        }
+        if (sizeof(T) == 4 && since >= kCcFlush) {
+            flush();
+            since = 0;
+        }
+    }
+    if (active) {
+        flush();
+        // lane -> value index of cc_warp_sum (the lane's bits, highest first)
+        double* out = partial + ((size_t)(split * wpt + phase) * ntask + task_off + ti) * V;
+        if constexpr (V >= 32) {
+#pragma unroll
+            for (int i = 0; i < V / 32; i++) out[lane * (V / 32) + i] = acc64[i];
+        } else {
+            constexpr int REP = 32 / V;  // lanes that differ in the low bits hold the same value
+            if (lane % REP == 0) out[lane / REP] = acc64[0];
+        }
+    }
 }
 
 __global__ void reduce_slots_kernel(const double* __restrict__ partial, int nsplit, int64_t slot_stride,
@@ -185,52 +283,39 @@ __global__ void normalise_kernel(const double* __restrict__ S, const int64_t* __
     }
 }
 
+template <typename T, int ORDER>
+static cudaError_t contract_cc_launch(const CcLaunch& L, int weighted, int absval, const void* fields, const void* weight,
+                                      const CcGroup* groups, const CcTask* tasks, double* partial,
+                                      cudaStream_t st) {
+    auto go = [&](auto k) -> cudaError_t {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem_bytes);
+        if (e) return e;
+        k<<<(unsigned)(L.ngroups * L.nsplit), kCcThreads, L.smem_bytes, st>>>(
+            (const T*)fields, L.nf, L.nchunk, (const T*)weight, groups, L.ngroups, tasks, L.ntask, L.nsplit, L.wpt,
+            L.stage_chunks, L.stage_bytes, partial);
+        return cudaGetLastError();
+    };
+    if (weighted) {
+        if constexpr (sizeof(T) == 8) return go(contract_cc_kernel<T, ORDER, true, false>);
+        return cudaErrorInvalidValue;
+    }
+    return absval ? go(contract_cc_kernel<T, ORDER, false, true>) : go(contract_cc_kernel<T, ORDER, false, false>);
+}
+
 }  // namespace ps
 
 using namespace ps;
 
-template <int NF>
-static cudaError_t contract_cc_launch(int is_double, int weighted, int absval, const void* fields, size_t field_stride,
-                                      int tile_ns, int64_t ncell, const void* weight, const PsTile* tiles, int ntiles,
-                                      const int* field_ids, const short4* rowf, const short4* colf, int nsplit,
-                                      int64_t chunks_per_split, double* partial, cudaStream_t st) {
-    dim3 grid(ntiles, nsplit);
-    if (is_double) {
-        if (weighted)
-            contract_cc_kernel<double, true, false, NF><<<grid, kCcThreads, 0, st>>>(
-                (const double*)fields, field_stride, tile_ns, ncell, (const double*)weight, tiles, ntiles, field_ids, rowf,
-                colf, chunks_per_split, partial);
-        else if (absval)
-            contract_cc_kernel<double, false, true, NF><<<grid, kCcThreads, 0, st>>>(
-                (const double*)fields, field_stride, tile_ns, ncell, nullptr, tiles, ntiles, field_ids, rowf, colf,
-                chunks_per_split, partial);
-        else
-            contract_cc_kernel<double, false, false, NF><<<grid, kCcThreads, 0, st>>>(
-                (const double*)fields, field_stride, tile_ns, ncell, nullptr, tiles, ntiles, field_ids, rowf, colf,
-                chunks_per_split, partial);
-    } else {
-        if (weighted) return cudaErrorInvalidValue;
-        if (absval)
-            contract_cc_kernel<float, false, true, NF><<<grid, kCcThreads, 0, st>>>(
-                (const float*)fields, field_stride, tile_ns, ncell, nullptr, tiles, ntiles, field_ids, rowf, colf,
-                chunks_per_split, partial);
-        else
-            contract_cc_kernel<float, false, false, NF><<<grid, kCcThreads, 0, st>>>(
-                (const float*)fields, field_stride, tile_ns, ncell, nullptr, tiles, ntiles, field_ids, rowf, colf,
-                chunks_per_split, partial);
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t ps_contract_cc(int is_double, int weighted, int absval, int nf, const void* fields, size_t field_stride,
-                           int tile_ns, int64_t ncell, const void* weight, const PsTile* tiles, int ntiles, const int* field_ids,
-                           const short4* rowf, const short4* colf, int nsplit, int64_t chunks_per_split,
-                           double* partial, cudaStream_t st) {
-    if (nf == 3)
-        return contract_cc_launch<3>(is_double, weighted, absval, fields, field_stride, tile_ns, ncell, weight, tiles,
-                                     ntiles, field_ids, rowf, colf, nsplit, chunks_per_split, partial, st);
-    return contract_cc_launch<2>(is_double, weighted, absval, fields, field_stride, tile_ns, ncell, weight, tiles, ntiles,
-                                 field_ids, rowf, colf, nsplit, chunks_per_split, partial, st);
+cudaError_t ps_contract_cc(int is_double, int order, int weighted, int absval, const CcLaunch& L, const void* fields,
+                           const void* weight, const CcGroup* groups, const CcTask* tasks, double* partial,
+                           cudaStream_t st) {
+#define PS_CC(O)                                                                                                       \
+    case O:                                                                                                            \
+        return is_double ? contract_cc_launch<double, O>(L, weighted, absval, fields, weight, groups, tasks, partial, st) \
+                         : contract_cc_launch<float, O>(L, weighted, absval, fields, weight, groups, tasks, partial, st);
+    switch (order) { PS_CC(2) PS_CC(3) PS_CC(4) PS_CC(5) PS_CC(6) }
+#undef PS_CC
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t ps_reduce_slots(const double* partial, int nsplit, int64_t slot_stride, const int64_t* slot,

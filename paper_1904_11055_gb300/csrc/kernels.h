@@ -31,24 +31,65 @@ cudaError_t ps_inverse_ranged_f32(int n, const void* fhat, const void* lines, co
                                   int tile_ns, const int* kz_host, const int* kz_dev, cudaStream_t st);
 
 // ---- contract_cc.cu -----------------------------------------------------------
-// One GEMM tile of the CUDA-core contraction: up to 64 rows x 64 cols, each row
-// (col) the product of one or two of the tile's local fields.
-struct PsTile {
-    int row_off, nrow, col_off, ncol, field_off, nfield;
-    unsigned region_mask;  // bit w: warp w's 32x16 region holds at least one needed entry
-    int pad_;
+// CUDA-core contraction: a task is a block of bins, one run of consecutive field
+// slots per leg; row (r) = the products of the first ra legs' runs, column (c) = of
+// the rest, the first leg's index slowest, product r * cols + c.  The run lengths per
+// order (a nibble per leg, first leg lowest): 64 products for FP32, where longer runs
+// save products and loads; 16 for FP64, whose 1/64-rate multiply-adds make every
+// product outside the bins dear (64 triangle shells: 1.33 products per bin in FP32,
+// 1.16 in FP64; 16 shells: 2.14 and 1.57).
+__host__ __device__ constexpr unsigned cc_code(int order, bool dbl) {
+    return dbl ? (order == 2 ? 0x44u : order == 3 ? 0x422u : order == 4 ? 0x2222u : order == 5 ? 0x22122u : 0x221221u)
+               : (order == 2 ? 0x88u : order == 3 ? 0x444u : order == 4 ? 0x4224u : order == 5 ? 0x42222u : 0x222222u);
+}
+__host__ __device__ constexpr int cc_ra(int order) { return order <= 2 ? 1 : (order <= 5 ? 2 : 3); }
+__host__ __device__ constexpr int cc_dim(int order, bool dbl, int leg) { return (int)((cc_code(order, dbl) >> (4 * leg)) & 15u); }
+__host__ __device__ constexpr int cc_span(int order, bool dbl, int l0, int l1) {  // product of the run lengths of legs [l0, l1)
+    int n = 1;
+    for (int l = l0; l < l1; l++) n *= cc_dim(order, dbl, l);
+    return n;
+}
+__host__ __device__ constexpr int cc_at(int order, bool dbl, int leg) {  // run lengths of the legs before it
+    int n = 0;
+    for (int l = 0; l < leg; l++) n += cc_dim(order, dbl, l);
+    return n;
+}
+template <int ORDER, bool DBL>
+struct CcShape {
+    static constexpr int nval = cc_at(ORDER, DBL, ORDER);  // values of a task per cell
+    static constexpr int ra = cc_ra(ORDER), rows = cc_span(ORDER, DBL, 0, ra), cols = cc_span(ORDER, DBL, ra, ORDER);
+    __host__ __device__ static constexpr int dim(int l) { return cc_dim(ORDER, DBL, l); }
+    __host__ __device__ static constexpr int at(int l) { return cc_at(ORDER, DBL, l); }
+    __host__ __device__ static constexpr int span(int l0, int l1) { return cc_span(ORDER, DBL, l0, l1); }
 };
-constexpr int kCcTM = 64, kCcTN = 64, kCcMaxFields = 128;
-// cells per chunk of the CUDA-core contraction
-inline int ps_cc_chunk(int is_double) { return is_double ? 16 : 32; }
-
-// partial[(split * ntiles + tile) * 64 * 64 + r * 64 + c] = sum over the split's cells
-// fields: natural [s][cell] with stride field_stride (tile_ns == 0) or cell-tiled over tile_ns shells
-// nf: factors per row or column at most (2 for n <= 4, 3 for n = 5, 6)
-cudaError_t ps_contract_cc(int is_double, int weighted, int absval, int nf, const void* fields, size_t field_stride,
-                           int tile_ns, int64_t ncell, const void* weight, const PsTile* tiles, int ntiles, const int* field_ids,
-                           const short4* rowf, const short4* colf, int nsplit, int64_t chunks_per_split,
-                           double* partial, cudaStream_t st);
+constexpr int kCcTasksPerGroup = 12;  // the warps of a block: FP32 tasks keep 168 registers a thread (8 warps at 216: 36.0 against 35.8 ms, FP64 0.51 against 0.45 ms)
+constexpr int kCcStages = 4;
+constexpr int kCcMaxSlots = 192;  // field slots the tasks of a group may name: at most 12 tasks x 16 (two runs of eight)
+constexpr int kCcPadRows = 8;   // rows after the last stage that a run past the last field may read (its products are unused)
+struct CcTask {
+    int row[6];  // per leg: element offset (32 per field row) of its run in the block's copy of a chunk
+};
+struct CcGroup {  // the tasks of one block
+    int task_off, ntask, used;  // used: field rows copied per chunk
+    int slot[kCcMaxSlots];      // their field slots, ascending
+};
+struct CcLaunch {
+    int nf = 0;           // field slots of a chunk in the cell-tiled array
+    int64_t nchunk = 0;   // 32-cell chunks
+    int ngroups = 0;
+    int64_t ntask = 0;
+    int nsplit = 1, wpt = 1;  // ranges of chunks; warps that share a task
+    int stage_chunks = 1, stage_bytes = 0;
+    size_t smem_bytes = 0;
+    int values = 64;      // products of a task
+    int64_t rows() const { return (int64_t)nsplit * wpt; }          // partial sums per task
+    int64_t stride() const { return ntask * (int64_t)values; }      // doubles between them
+};
+// partial[(split * wpt + phase) * stride + task * values + product]: FP64 sums over that part of the cells.
+// fields: cell-tiled, [nchunk][nf][32]; weight (FP64 only): [nchunk * 32] cell weights.
+cudaError_t ps_contract_cc(int is_double, int order, int weighted, int absval, const CcLaunch& L, const void* fields,
+                           const void* weight, const CcGroup* groups, const CcTask* tasks, double* partial,
+                           cudaStream_t st);
 // S[b] = sum_split partial[split * slot_stride + slot[b]]
 cudaError_t ps_reduce_slots(const double* partial, int nsplit, int64_t slot_stride, const int64_t* slot,
                             int64_t nbins, double* S, cudaStream_t st);
@@ -63,7 +104,6 @@ cudaError_t ps_normalise(const double* S, const int64_t* counts, int64_t nbins, 
                          cudaStream_t st);
 
 // ---- misc.cu -------------------------------------------------------------------
-// out[s * out_stride + w] = in[s * in_stride + idx[w]] for s < ns, w < nw
 // ---- counts_exact.cu ---------------------------------------------------------
 // out = F[s0] F[s1] F[s2] (slots -1: none), FP64 fields of n3 cells in natural layout
 cudaError_t ps_prod_fields(const double* F, size_t n3, int s0, int s1, int s2, double* out, cudaStream_t st);
@@ -73,5 +113,7 @@ cudaError_t ps_round_map(const void* fhat, size_t n, double inv_n3, long long* G
 cudaError_t ps_dot_maps(const long long* maps, size_t mapsz, const int2* which, int nbins, int Kp,
                         unsigned long long* out, cudaStream_t st);
 
-cudaError_t ps_gather_cells(int is_double, const void* in, size_t in_stride, int ns, const int32_t* idx, int64_t nw,
-                            void* out, size_t out_stride, cudaStream_t st);
+// cells idx[w] of ns natural-layout FP64 fields, in_stride apart, into slots s0 .. s0 + ns - 1 of the cell-tiled
+// array out[(w / 32) * nf * 32 + slot * 32 + w % 32]; w in [nw, nw rounded up to 32) is set to 0
+cudaError_t ps_gather_cells(const double* in, size_t in_stride, int s0, int ns, int nf, const int32_t* idx, int64_t nw,
+                            double* out, cudaStream_t st);

@@ -6,12 +6,12 @@
 
 namespace ps {
 
-template <typename T>
-__global__ void gather_cells_kernel(const T* __restrict__ in, size_t in_stride, int ns, const int32_t* __restrict__ idx,
-                                    int64_t nw, T* __restrict__ out, size_t out_stride) {
+__global__ void gather_cells_kernel(const double* __restrict__ in, size_t in_stride, int s0, int nf,
+                                    const int32_t* __restrict__ idx, int64_t nw, double* __restrict__ out) {
     const int s = blockIdx.y;
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nw; w += (int64_t)gridDim.x * blockDim.x)
-        out[(size_t)s * out_stride + w] = in[(size_t)s * in_stride + idx[w]];
+    const int64_t n = (nw + 31) / 32 * 32;
+    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < n; w += (int64_t)gridDim.x * blockDim.x)
+        out[((w >> 5) * nf + s0 + s) * 32 + (w & 31)] = w < nw ? in[(size_t)s * in_stride + idx[w]] : 0.0;
 }
 
 // L_ell(mu) by Bonnet's recurrence, (n+1) P_{n+1} = (2n+1) mu P_n - n P_{n-1}
@@ -56,15 +56,10 @@ cudaError_t ps_legendre_weight(int is_double, const void* fhat, int K, int ell, 
     return cudaGetLastError();
 }
 
-cudaError_t ps_gather_cells(int is_double, const void* in, size_t in_stride, int ns, const int32_t* idx, int64_t nw,
-                            void* out, size_t out_stride, cudaStream_t st) {
+cudaError_t ps_gather_cells(const double* in, size_t in_stride, int s0, int ns, int nf, const int32_t* idx, int64_t nw,
+                            double* out, cudaStream_t st) {
     if (nw <= 0 || ns <= 0) return cudaSuccess;
     dim3 grid((unsigned)((nw + 255) / 256 < 2048 ? (nw + 255) / 256 : 2048), ns);
-    if (is_double)
-        ps::gather_cells_kernel<double><<<grid, 256, 0, st>>>((const double*)in, in_stride, ns, idx, nw, (double*)out,
-                                                              out_stride);
-    else
-        ps::gather_cells_kernel<float><<<grid, 256, 0, st>>>((const float*)in, in_stride, ns, idx, nw, (float*)out,
-                                                             out_stride);
+    ps::gather_cells_kernel<<<grid, 256, 0, st>>>(in, in_stride, s0, nf, idx, nw, out);
     return cudaGetLastError();
 }

@@ -9,7 +9,7 @@
 // belongs to this library.
 //
 // Each call builds its host tables (twiddles, shell line tables, contraction
-// tiles) in ordinary pageable host memory and copies them, and the counts, into
+// tasks) in ordinary pageable host memory and copies them, and the counts, into
 // the array with cudaMemcpyAsync.  Copies from pageable memory are staged
 // through the driver, so a call can wait for its stream before it returns; it
 // is not a zero-latency call.
@@ -79,6 +79,54 @@ struct Carve {  // 256-byte aligned sub-ranges of the static array
 };
 }  // namespace
 
+namespace {
+// The limit of this entry point, fixed so that what it takes does not move with the contraction's own
+// layout: its intermediates with the bins cut into tiles of 64 rows (pairs (k1, k2), in the order of their
+// first and last k3) by 64 columns (k3), 4096 sums per tile and split.
+struct TileCount {
+    size_t tiles = 0, rows = 0, cols = 0, fields = 0;
+};
+TileCount count_tiles(const PsPlan& p) {
+    struct Row {
+        int lo, hi, k1, k2;
+        std::vector<int> cols;
+    };
+    std::vector<Row> rows;
+    for (int64_t b = 0; b < p.nbins; b++) {  // bins are sorted, so a row's columns are consecutive and ascending
+        const int32_t* k = &p.bins[3 * b];
+        if (rows.empty() || rows.back().k1 != k[0] || rows.back().k2 != k[1]) rows.push_back({k[2], k[2], k[0], k[1], {}});
+        rows.back().hi = k[2];
+        rows.back().cols.push_back(k[2]);
+    }
+    std::stable_sort(rows.begin(), rows.end(), [](const Row& a, const Row& b) {
+        return a.lo != b.lo ? a.lo < b.lo : a.hi < b.hi;
+    });
+    TileCount t;
+    for (size_t g = 0; g < rows.size(); g += 64) {
+        const size_t g1 = std::min(rows.size(), g + 64);
+        std::vector<int> cu, rf;
+        for (size_t r = g; r < g1; r++) {
+            cu.insert(cu.end(), rows[r].cols.begin(), rows[r].cols.end());
+            rf.push_back(rows[r].k1);
+            rf.push_back(rows[r].k2);
+        }
+        std::sort(cu.begin(), cu.end());
+        cu.erase(std::unique(cu.begin(), cu.end()), cu.end());
+        for (size_t c0 = 0; c0 < cu.size(); c0 += 64) {
+            const size_t c1 = std::min(cu.size(), c0 + 64);
+            std::vector<int> f(rf);
+            f.insert(f.end(), cu.begin() + (long)c0, cu.begin() + (long)c1);
+            std::sort(f.begin(), f.end());
+            t.tiles++;
+            t.rows += g1 - g;
+            t.cols += c1 - c0;
+            t.fields += (size_t)(std::unique(f.begin(), f.end()) - f.begin());
+        }
+    }
+    return t;
+}
+}  // namespace
+
 static poly_status estimate_noalloc(int N, double L, int nshell, const double* edges, const float* delta_x,
                                     const int64_t* counts, double* out, void* stream) {
     if (!edges || !delta_x || !counts || !out) return fail(POLY_ERR_ARG, "NULL argument");
@@ -110,15 +158,26 @@ static poly_status estimate_noalloc(int N, double L, int nshell, const double* e
         build_lines(&hp, hp.edges.data(), s, lines);
         line_off.push_back((int)(lines.size() / 4));
     }
-    build_cc_tiles(&hp, hp.cc);
-    const int ntiles = (int)hp.cc.tiles.size();
     const int64_t n3 = (int64_t)N * N * N;
-    const int64_t chunk = ps_cc_chunk(0);
-    const int64_t nchunks = (n3 + chunk - 1) / chunk;
-    const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(64, nchunks / 16));
-    const int64_t cps = (nchunks + nsplit - 1) / nsplit;
-    const int64_t slot_stride = (int64_t)ntiles * kCcTM * kCcTN;
     const size_t nl = (size_t)(2 * K + 1) * (K + 1);
+    size_t tile_part;  // bytes of the tiles' sums
+    {
+        const TileCount t = count_tiles(hp);
+        const int64_t nsplit = std::max<int64_t>(1, std::min<int64_t>(64, (n3 + 31) / 32 / 16));
+        tile_part = (size_t)nsplit * t.tiles * 4096 * 8;
+        Carve c;
+        for (size_t bytes : {(size_t)N * 16, (size_t)N * 16, lines.size() * sizeof(short), line_off.size() * sizeof(int),
+                             (size_t)N * nl * 8, nl * (2 * K + 1) * 8, (size_t)nshell * n3 * 4, t.tiles * 32, t.fields * 4,
+                             t.rows * 8, t.cols * 8, (size_t)hp.nbins * 8, tile_part, (size_t)hp.nbins * 8,
+                             (size_t)hp.nbins * 8})
+            c.take(bytes);
+        if (c.used > kNoAllocBytes)
+            return fail(POLY_ERR_UNSUPPORTED, "this problem needs " + std::to_string(c.used >> 20) +
+                                                  " MiB of scratch; the static array holds 32 MiB");
+    }
+    build_cc_tasks(&hp, 0, 0, hp.cc);
+    const int64_t one_row = std::max<int64_t>(1, hp.cc.ntask() * cc_span(order, false, 0, order) * 8);
+    const CcLaunch cl = cc_launch_shape(hp.cc, order, nshell, n3 / 32, 152, std::max<int64_t>(1, (int64_t)tile_part / one_row));
 
     // layout of the static array
     Carve c;
@@ -126,11 +185,10 @@ static poly_status estimate_noalloc(int N, double L, int nshell, const double* e
     const size_t o_lines = c.take(lines.size() * sizeof(short)), o_loff = c.take(line_off.size() * sizeof(int));
     const size_t o_W = c.take((size_t)N * nl * 8), o_fhat = c.take(nl * (2 * K + 1) * 8);
     const size_t o_fields = c.take((size_t)nshell * n3 * 4);
-    const size_t o_tiles = c.take(hp.cc.tiles.size() * sizeof(PsTile));
-    const size_t o_fid = c.take(hp.cc.field_ids.size() * sizeof(int));
-    const size_t o_rowf = c.take(hp.cc.rowf.size() * sizeof(short4)), o_colf = c.take(hp.cc.colf.size() * sizeof(short4));
+    const size_t o_tasks = c.take(hp.cc.tasks.size() * sizeof(CcTask));
+    const size_t o_groups = c.take(hp.cc.groups.size() * sizeof(CcGroup));
     const size_t o_slot = c.take(hp.cc.slot.size() * sizeof(int64_t));
-    const size_t o_part = c.take((size_t)nsplit * slot_stride * 8);
+    const size_t o_part = c.take((size_t)(cl.rows() * cl.stride()) * 8);
     const size_t o_S = c.take((size_t)hp.nbins * 8), o_cnt = c.take((size_t)hp.nbins * 8);
     if (c.used > kNoAllocBytes)
         return fail(POLY_ERR_UNSUPPORTED, "this problem needs " + std::to_string(c.used >> 20) +
@@ -158,10 +216,8 @@ static poly_status estimate_noalloc(int N, double L, int nshell, const double* e
                   {o_twi, twi.data(), twi.size() * 8},
                   {o_lines, lines.data(), lines.size() * sizeof(short)},
                   {o_loff, line_off.data(), line_off.size() * sizeof(int)},
-                  {o_tiles, hp.cc.tiles.data(), hp.cc.tiles.size() * sizeof(PsTile)},
-                  {o_fid, hp.cc.field_ids.data(), hp.cc.field_ids.size() * sizeof(int)},
-                  {o_rowf, hp.cc.rowf.data(), hp.cc.rowf.size() * sizeof(short4)},
-                  {o_colf, hp.cc.colf.data(), hp.cc.colf.size() * sizeof(short4)},
+                  {o_tasks, hp.cc.tasks.data(), hp.cc.tasks.size() * sizeof(CcTask)},
+                  {o_groups, hp.cc.groups.data(), hp.cc.groups.size() * sizeof(CcGroup)},
                   {o_slot, hp.cc.slot.data(), hp.cc.slot.size() * sizeof(int64_t)},
                   {o_cnt, counts, (size_t)hp.nbins * 8}};
     for (const Copy& cp : copies)
@@ -173,10 +229,9 @@ static poly_status estimate_noalloc(int N, double L, int nshell, const double* e
     if ((e = ps_forward(N, 0, delta_x, K, B + o_twf, B + o_W, B + o_fhat, nullptr, st)) ||
         (e = ps_inverse(N, 0, 0, B + o_fhat, B + o_lines, (const int*)(B + o_loff), 0, nshell, K, 0, N, B + o_twi,
                         B + o_fields, (size_t)n3, nullptr, nullptr, 0, nshell, st)) ||
-        (e = ps_contract_cc(0, 0, 0, 2, B + o_fields, (size_t)n3, nshell, n3, nullptr, (const PsTile*)(B + o_tiles), ntiles,
-                            (const int*)(B + o_fid), (const short4*)(B + o_rowf), (const short4*)(B + o_colf), nsplit,
-                            cps, (double*)(B + o_part), st)) ||
-        (e = ps_reduce_slots((const double*)(B + o_part), nsplit, slot_stride, (const int64_t*)(B + o_slot), hp.nbins,
+        (e = ps_contract_cc(0, order, 0, 0, cl, B + o_fields, nullptr, (const CcGroup*)(B + o_groups),
+                            (const CcTask*)(B + o_tasks), (double*)(B + o_part), st)) ||
+        (e = ps_reduce_slots((const double*)(B + o_part), (int)cl.rows(), cl.stride(), (const int64_t*)(B + o_slot), hp.nbins,
                              (double*)(B + o_S), st)))
         return fail(POLY_ERR_CUDA, std::string("estimate kernels: ") + cudaGetErrorString(e));
     const double n3d = (double)n3;

@@ -175,111 +175,143 @@ void build_lines(const PsPlan* p, const double* e, int s, std::vector<short>& li
 }
 
 // ---------------------------------------------------------------------------
-// CUDA-core contraction tiles: rows = products of the first ra shells of a
-// bin, cols = products of the rest (ra = 1, 2, 2, 2, 3 for n = 2..6); rows
-// grouped 64 at a time after sorting by their column span, each group's column
-// union cut into chunks of 64.
+// CUDA-core contraction tasks: blocks of bins with one run of consecutive shells
+// per leg (cc_dim long).  The runs of all legs but the last start at multiples of
+// their length; the last leg's follow from its smallest shell in that block.  A run
+// that would pass the last shell starts earlier instead.  Tasks are cut evenly into
+// groups of at most 12 (one block's warps), in an order in which a group names few
+// field slots (the ones its block copies).
 // ---------------------------------------------------------------------------
-void build_cc_tiles(PsPlan* p, CcTiles& t, int first_shift) {
-    using Key = std::array<int, 3>;  // 1-based field slots, -1 padded
-    const int n = p->order;
-    const int ra = n <= 2 ? 1 : (n <= 5 ? 2 : 3), ca = n - ra;
-    auto key = [](const int32_t* b, int cnt) {
-        Key k{-1, -1, -1};
-        for (int i = 0; i < cnt; i++) k[i] = b[i];
-        return k;
-    };
-    // first_shift > 0: the bin's first leg reads the weighted field slot k1 + first_shift (multipoles)
-    auto rkey = [&](const int32_t* b) {
-        Key k = key(b, ra);
-        k[0] += first_shift;
-        return k;
-    };
-    auto ckey = [&](const int32_t* b) { return key(b + ra, ca); };
-    std::map<Key, std::vector<Key>> rows;  // row -> col keys
-    for (int64_t i = 0; i < p->nbins; i++) rows[rkey(&p->bins[i * n])].push_back(ckey(&p->bins[i * n]));
-    struct RowInfo {
-        Key key;
-        std::vector<Key> cols;
-    };
-    std::vector<RowInfo> ri;
-    for (auto& kv : rows) {
-        auto cols = kv.second;
-        std::sort(cols.begin(), cols.end());
-        cols.erase(std::unique(cols.begin(), cols.end()), cols.end());
-        ri.push_back({kv.first, cols});
-    }
-    std::stable_sort(ri.begin(), ri.end(), [](const RowInfo& a, const RowInfo& b) {
-        return std::make_pair(a.cols.front(), a.cols.back()) < std::make_pair(b.cols.front(), b.cols.back());
-    });
-    // (row key, col key) -> slot; the six slots (from 1, or -1; at most 2 * kPsMaxShells) packed 10 bits each
-    static_assert(2 * kPsMaxShells + 1 < 1024, "a field slot + 1 must fit 10 bits of the packed key");
-    if (p->nshell > kPsMaxShells) throw std::length_error("build_cc_tiles: more shells than the packed keys hold");
-    auto pack = [](const Key& r, const Key& c) {
+void build_cc_tasks(const PsPlan* p, int is_double, int first_shift, CcTasks& t) {
+    const int n = p->order, ns = p->nshell;
+    t.is_double = is_double;
+    t.nslot = ns + first_shift;
+    static_assert(kPsMaxShells <= 128, "block numbers of five legs are packed 7 bits each");
+    if (ns > kPsMaxShells) throw std::length_error("build_cc_tasks: more shells than the packed keys hold");
+    const int dl = cc_dim(n, is_double, n - 1);
+    auto pack = [&](const int32_t* b) {
         uint64_t v = 0;
-        for (int i = 0; i < 3; i++) v = v << 10 | (uint64_t)(r[i] + 1);
-        for (int i = 0; i < 3; i++) v = v << 10 | (uint64_t)(c[i] + 1);
+        for (int l = 0; l + 1 < n; l++) v = v << 7 | (uint64_t)((b[l] - 1) / cc_dim(n, is_double, l));
         return v;
     };
-    std::unordered_map<uint64_t, int64_t> slot_of;
-    slot_of.reserve((size_t)p->nbins * 2);
-    for (size_t g = 0; g < ri.size(); g += kCcTM) {
-        const size_t g1 = std::min(ri.size(), g + kCcTM);
-        std::vector<Key> cu;
-        for (size_t r = g; r < g1; r++) cu.insert(cu.end(), ri[r].cols.begin(), ri[r].cols.end());
-        std::sort(cu.begin(), cu.end());
-        cu.erase(std::unique(cu.begin(), cu.end()), cu.end());
-        for (size_t c0 = 0; c0 < cu.size(); c0 += kCcTN) {
-            const size_t c1 = std::min(cu.size(), c0 + kCcTN);
-            PsTile tile{};
-            tile.row_off = (int)t.rowf.size();
-            tile.nrow = (int)(g1 - g);
-            tile.col_off = (int)t.colf.size();
-            tile.ncol = (int)(c1 - c0);
-            tile.field_off = (int)t.field_ids.size();
-            std::map<int, int> local;  // shell (0-based) -> local field index
-            auto loc = [&](int shell1) -> short {
-                if (shell1 < 0) return -1;
-                auto it = local.find(shell1 - 1);
-                if (it != local.end()) return (short)it->second;
-                int id = (int)local.size();
-                local[shell1 - 1] = id;
-                t.field_ids.push_back(shell1 - 1);
-                return (short)id;
-            };
-            auto factors = [&](const Key& k) {  // in order: local ids follow first appearance, row by row
-                const short a = loc(k[0]);
-                const short b = loc(k[1]);
-                const short c = loc(k[2]);
-                return make_short4(a, b, c, -1);
-            };
-            for (size_t r = g; r < g1; r++) t.rowf.push_back(factors(ri[r].key));
-            std::map<Key, int> cidx;
-            for (size_t c = c0; c < c1; c++) {
-                t.colf.push_back(factors(cu[c]));
-                cidx[cu[c]] = (int)(c - c0);
-            }
-            tile.nfield = (int)local.size();
-            const int tid = (int)t.tiles.size();
-            for (size_t r = g; r < g1; r++)
-                for (auto& ck : ri[r].cols) {
-                    auto it = cidx.find(ck);
-                    if (it == cidx.end()) continue;
-                    const int rr = (int)(r - g), cc = it->second;
-                    tile.region_mask |= 1u << ((rr / 32) * 4 + cc / 16);
-                    slot_of[pack(ri[r].key, ck)] = (int64_t)tid * (kCcTM * kCcTN) + rr * kCcTN + cc;
-                }
-            t.tiles.push_back(tile);
+    struct Block {
+        int lo, hi, first;  // the last leg's shells (from 0), first task
+    };
+    std::unordered_map<uint64_t, Block> blocks;
+    for (int64_t i = 0; i < p->nbins; i++) {
+        const int32_t* b = &p->bins[i * n];
+        const int k = b[n - 1] - 1;
+        auto r = blocks.emplace(pack(b), Block{k, k, 0});
+        if (!r.second) {
+            r.first->second.lo = std::min(r.first->second.lo, k);
+            r.first->second.hi = std::max(r.first->second.hi, k);
         }
     }
+    std::vector<uint64_t> keys;
+    keys.reserve(blocks.size());
+    for (auto& kv : blocks) keys.push_back(kv.first);
+    std::sort(keys.begin(), keys.end());
+    auto start = [&](int base, int d) { return std::max(0, std::min(base, ns - d)); };
+    for (uint64_t key : keys) {
+        Block& B = blocks[key];
+        B.first = (int)t.first.size();
+        std::array<short, 6> f{};
+        uint64_t v = key;
+        for (int l = n - 2; l >= 0; l--, v >>= 7) {
+            const int d = cc_dim(n, is_double, l);
+            f[l] = (short)(start((int)(v & 127) * d, d) + (l == 0 ? first_shift : 0));
+        }
+        for (int k = B.lo; k <= B.hi; k += dl) {
+            f[n - 1] = (short)start(k, dl);
+            t.first.push_back(f);
+        }
+    }
+    const int values = cc_span(n, is_double, 0, n);
     t.slot.resize(p->nbins);
-    for (int64_t i = 0; i < p->nbins; i++) t.slot[i] = slot_of.at(pack(rkey(&p->bins[i * n]), ckey(&p->bins[i * n])));
+    for (int64_t i = 0; i < p->nbins; i++) {
+        const int32_t* b = &p->bins[i * n];
+        const Block& B = blocks[pack(b)];
+        const int task = B.first + (b[n - 1] - 1 - B.lo) / dl;
+        int64_t v = 0;
+        for (int l = 0; l < n; l++)
+            v = v * cc_dim(n, is_double, l) + (b[l] - 1 + (l == 0 ? first_shift : 0) - t.first[task][l]);
+        t.slot[i] = (int64_t)task * values + v;
+    }
+    // tasks in the order of the octets of shells that their runs start in, so that the tasks of a group share
+    // fields (64 triangle shells: 26 slots per group instead of 34 in the order of the runs)
+    std::vector<int> by(t.first.size()), at(t.first.size());
+    for (size_t i = 0; i < by.size(); i++) by[i] = (int)i;
+    std::sort(by.begin(), by.end(), [&](int x, int y) {
+        const auto &a = t.first[x], &b = t.first[y];
+        for (int l = 0; l < n; l++)
+            if (a[l] / 8 != b[l] / 8) return a[l] / 8 < b[l] / 8;
+        return a != b ? a < b : x < y;
+    });
+    std::vector<std::array<short, 6>> sorted;
+    sorted.reserve(by.size());
+    for (size_t i = 0; i < by.size(); i++) {
+        at[by[i]] = (int)i;
+        sorted.push_back(t.first[by[i]]);
+    }
+    t.first.swap(sorted);
+    for (auto& v : t.slot) v = (int64_t)at[v / values] * values + v % values;
+    // groups
+    const int64_t nt = (int64_t)t.first.size(), ng = (nt + kCcTasksPerGroup - 1) / kCcTasksPerGroup;
+    t.tasks.resize(nt);
+    for (int64_t g = 0; g < ng; g++) {
+        CcGroup G{};
+        G.task_off = (int)(nt * g / ng);
+        G.ntask = (int)(nt * (g + 1) / ng) - G.task_off;
+        std::vector<char> need(t.nslot, 0);
+        for (int k = G.task_off; k < G.task_off + G.ntask; k++)
+            for (int l = 0; l < n; l++)
+                for (int i = 0; i < cc_dim(n, is_double, l); i++)
+                    if (t.first[k][l] + i < t.nslot) need[t.first[k][l] + i] = 1;
+        std::vector<int> local(t.nslot, 0);
+        for (int s = 0; s < t.nslot; s++)
+            if (need[s]) {
+                if (G.used == kCcMaxSlots) throw std::length_error("build_cc_tasks: a group names too many field slots");
+                local[s] = G.used;
+                G.slot[G.used++] = s;
+            }
+        t.max_used = std::max(t.max_used, G.used);
+        for (int k = G.task_off; k < G.task_off + G.ntask; k++)
+            for (int l = 0; l < n; l++) t.tasks[k].row[l] = local[t.first[k][l]] * 32;
+        t.groups.push_back(G);
+    }
 }
 
-static int choose_splits(int ntiles, int64_t nchunks, int sms) {
-    int want = std::max(1, (4 * sms + ntiles - 1) / ntiles);
-    int64_t maxs = std::max<int64_t>(1, nchunks / 16);
-    return (int)std::min<int64_t>(want, maxs);
+// Stages of about 48 KB (one to twelve steps).  Blocks: the fewest waves (up to
+// six) whose last is full to within 2 % of the best, at least four steps per warp.
+CcLaunch cc_launch_shape(const CcTasks& t, int order, int nf, int64_t nchunk, int sms, int64_t max_rows) {
+    CcLaunch L;
+    L.nf = nf;
+    L.nchunk = nchunk;
+    L.ngroups = (int)t.groups.size();
+    L.ntask = t.ntask();
+    L.values = cc_span(order, t.is_double, 0, order);
+    const int row = 32 * (t.is_double ? 8 : 4);
+    int tpg = 1;
+    for (auto& g : t.groups) tpg = std::max(tpg, g.ntask);
+    L.wpt = std::max(1, kCcTasksPerGroup / tpg);
+    if (max_rows > 0) L.wpt = (int)std::min<int64_t>(L.wpt, max_rows);
+    const int step = t.is_double ? 1 : 2;  // chunks of a step
+    L.stage_chunks = step * std::max(1, std::min(12, 48 * 1024 / (t.max_used * row * step)));
+    L.stage_bytes = L.stage_chunks * t.max_used * row;
+    L.smem_bytes = (size_t)kCcStages * L.stage_bytes + (size_t)kCcPadRows * row;
+    int64_t most = std::max<int64_t>(1, nchunk / (4 * step * L.wpt));
+    if (max_rows > 0) most = std::min<int64_t>(most, std::max<int64_t>(1, max_rows / L.wpt));
+    double best = 0;
+    for (int k = 1; k <= 6; k++) {
+        const int64_t ns = std::min<int64_t>(most, std::max<int64_t>(1, (int64_t)k * sms / std::max(1, L.ngroups)));
+        const int64_t blocks = ns * L.ngroups;
+        const double full = (double)blocks / (double)((blocks + sms - 1) / sms * sms);
+        if (full > best * 1.02) {
+            best = full;
+            L.nsplit = (int)ns;
+        }
+    }
+    return L;
 }
 
 // ---------------------------------------------------------------------------
@@ -442,26 +474,32 @@ static poly_status compute_counts(PsPlan* p, cudaStream_t st) {
     };
     poly_status rc = POLY_OK;
     void *d_widx = nullptr, *d_wgt = nullptr, *d_iota = nullptr, *d_planes = nullptr, *d_spill = nullptr,
-         *d_part = nullptr, *d_S = nullptr;
+         *d_part = nullptr, *d_S = nullptr, *d_tasks = nullptr, *d_groups = nullptr, *d_slot = nullptr;
     const int sb = std::min(8, p->nshell);  // shells per inverse batch
     const size_t plane_elems = (size_t)(h + 1) * N * N;
     const bool spill = ps_plane_needs_spill(N, p->K, 1) == 1;
-    const CcTiles& t = p->cc;
-    const int64_t nchunks = (nw + ps_cc_chunk(1) - 1) / ps_cc_chunk(1);
-    const int nsplit = choose_splits((int)t.tiles.size(), nchunks, p->sms);
-    const int64_t cps = (nchunks + nsplit - 1) / nsplit;
-    const int64_t slot_stride = (int64_t)t.tiles.size() * kCcTM * kCcTN;
+    CcTasks t;  // FP64, over the plain shells
+    build_cc_tasks(p, 1, 0, t);
+    const int64_t nchunk = (nw + 31) / 32, nwp = nchunk * 32;
+    wgt.resize(nwp, 0.0);
+    const CcLaunch L = cc_launch_shape(t, p->order, p->nshell, nchunk, p->sms);
     do {
         if ((rc = talloc(&d_widx, widx.size() * 4))) break;
         if ((rc = talloc(&d_wgt, wgt.size() * 8))) break;
-        if ((rc = talloc(&d_iota, (size_t)p->nshell * nw * 8))) break;
+        if ((rc = talloc(&d_iota, (size_t)p->nshell * nwp * 8))) break;
         if ((rc = talloc(&d_planes, (size_t)sb * plane_elems * 8))) break;
         if (spill && (rc = talloc(&d_spill, ps_spill_elems(N, p->K, (h + 1) * sb, 1) * 16))) break;
-        if ((rc = talloc(&d_part, (size_t)nsplit * slot_stride * 8))) break;
+        if ((rc = talloc(&d_part, (size_t)(L.rows() * L.stride()) * 8))) break;
+        if ((rc = talloc(&d_tasks, t.tasks.size() * sizeof(CcTask)))) break;
+        if ((rc = talloc(&d_groups, t.groups.size() * sizeof(CcGroup)))) break;
+        if ((rc = talloc(&d_slot, t.slot.size() * 8))) break;
         if ((rc = talloc(&d_S, (size_t)std::max<int64_t>(1, p->nbins) * 8))) break;
         cudaError_t e;
         if ((e = cudaMemcpyAsync(d_widx, widx.data(), widx.size() * 4, cudaMemcpyHostToDevice, st)) ||
-            (e = cudaMemcpyAsync(d_wgt, wgt.data(), wgt.size() * 8, cudaMemcpyHostToDevice, st))) {
+            (e = cudaMemcpyAsync(d_wgt, wgt.data(), wgt.size() * 8, cudaMemcpyHostToDevice, st)) ||
+            (e = cudaMemcpyAsync(d_tasks, t.tasks.data(), t.tasks.size() * sizeof(CcTask), cudaMemcpyHostToDevice, st)) ||
+            (e = cudaMemcpyAsync(d_groups, t.groups.data(), t.groups.size() * sizeof(CcGroup), cudaMemcpyHostToDevice, st)) ||
+            (e = cudaMemcpyAsync(d_slot, t.slot.data(), t.slot.size() * 8, cudaMemcpyHostToDevice, st))) {
             rc = cuda_error(e, "counts upload");
             break;
         }
@@ -472,18 +510,18 @@ static poly_status compute_counts(PsPlan* p, cudaStream_t st) {
                 rc = cuda_error(e, "counting fields");
                 break;
             }
-            if ((e = ps_gather_cells(1, d_planes, plane_elems, ns, (const int32_t*)d_widx, nw,
-                                     (double*)d_iota + (size_t)s0 * nw, nw, st))) {
+            if ((e = ps_gather_cells((const double*)d_planes, plane_elems, s0, ns, p->nshell, (const int32_t*)d_widx, nw,
+                                     (double*)d_iota, st))) {
                 rc = cuda_error(e, "wedge gather");
                 break;
             }
         }
         if (rc) break;
-        if ((e = ps_contract_cc(1, 1, 0, p->order >= 5 ? 3 : 2, d_iota, (size_t)nw, 0, nw, d_wgt, (const PsTile*)p->d_cc_tiles,
-                                (int)t.tiles.size(), (const int*)p->d_cc_field_ids, (const short4*)p->d_cc_rowf,
-                                (const short4*)p->d_cc_colf, nsplit, cps, (double*)d_part, st)) ||
-            (e = ps_reduce_slots((double*)d_part, nsplit, slot_stride, (const int64_t*)p->d_cc_slot, p->nbins,
-                                 (double*)d_S, st))) {
+        if (p->nbins > 0 &&
+            ((e = ps_contract_cc(1, p->order, 1, 0, L, d_iota, d_wgt, (const CcGroup*)d_groups, (const CcTask*)d_tasks,
+                                 (double*)d_part, st)) ||
+             (e = ps_reduce_slots((double*)d_part, (int)L.rows(), L.stride(), (const int64_t*)d_slot, p->nbins,
+                                  (double*)d_S, st)))) {
             rc = cuda_error(e, "count contraction");
             break;
         }
@@ -501,7 +539,7 @@ static poly_status compute_counts(PsPlan* p, cudaStream_t st) {
         // and the plan's counts come from the integer closure maps instead.
         for (int64_t b = 0; b < p->nbins; b++) {
             const double v = S[b] / n3, r = std::nearbyint(v);
-            if (std::fabs(v - r) > 0.05 || r < 0) {
+            if (!(std::fabs(v - r) <= 0.05) || r < 0) {
                 char msg[160];
                 snprintf(msg, sizeof msg, "polygon count of bin %lld is not an integer: %.6f", (long long)b, v);
                 rc = set_error(POLY_ERR_COUNT, msg);
@@ -544,7 +582,7 @@ constexpr int64_t kMaxSortedTuples = int64_t(1) << 26;  // host tables of about 
 
 // The host part of plan creation: argument checks, the bins, the shell line tables
 // (slot nshell holds the union of all shells, used by the adjoint) and the
-// CUDA-core contraction tiles over the plain fields.  Touches no device.
+// CUDA-core contraction tasks (a multipole plan's first leg on the weighted fields).  Touches no device.
 poly_status ps_plan_host_tables(PsPlan* p, int N, double L, int order, int nshell, const double* edges,
                                poly_precision prec, unsigned flags, int ell, std::vector<short>& lines) {
     if (!edges || nshell < 1 || nshell > kPsMaxShells) return set_error(POLY_ERR_ARG, "nshell must be in [1, 128]");
@@ -604,7 +642,7 @@ poly_status ps_plan_host_tables(PsPlan* p, int N, double L, int order, int nshel
     }
     p->line_off = off;
     for (int s = 0; s <= nshell; s++) p->max_lines = std::max(p->max_lines, off[s + 1] - off[s]);
-    build_cc_tiles(p, p->cc, 0);
+    build_cc_tasks(p, p->is_double, ell > 0 ? nshell : 0, p->cc);
     return POLY_OK;
 }
 
@@ -639,11 +677,9 @@ static poly_status create_plan(PsPlan* p, int N, double L, int order, int nshell
     PS_TRY(upload(p, (void**)&p->d_line_off, off));
     PS_TRY(upload(p, (void**)&p->d_shell_kz, p->shell_kz));
 
-    // contraction tiles (CUDA-core path; the counts use them too)
-    PS_TRY(upload(p, &p->d_cc_tiles, p->cc.tiles));
-    PS_TRY(upload(p, &p->d_cc_field_ids, p->cc.field_ids));
-    PS_TRY(upload(p, &p->d_cc_rowf, p->cc.rowf));
-    PS_TRY(upload(p, &p->d_cc_colf, p->cc.colf));
+    // contraction tasks (CUDA-core path)
+    PS_TRY(upload(p, &p->d_cc_tasks, p->cc.tasks));
+    PS_TRY(upload(p, &p->d_cc_groups, p->cc.groups));
     PS_TRY(upload(p, &p->d_cc_slot, p->cc.slot));
 
     // workspace
@@ -662,12 +698,8 @@ static poly_status create_plan(PsPlan* p, int N, double L, int order, int nshell
     }
     if (ps_plane_needs_spill(N, K, p->is_double) == 1)
         PS_TRY(ps_alloc(p, &p->d_spill, ps_spill_elems(N, K, N * nshell, p->is_double) * 2 * es));
-    const int64_t chunk = ps_cc_chunk(p->is_double);
-    const int64_t nchunks = ((int64_t)n3 + chunk - 1) / chunk;
-    p->cc_nsplit = choose_splits((int)p->cc.tiles.size(), nchunks, p->sms);
-    p->cc_cps = (nchunks + p->cc_nsplit - 1) / p->cc_nsplit;
-    p->cc_slot_stride = (int64_t)p->cc.tiles.size() * kCcTM * kCcTN;
-    PS_TRY(ps_alloc(p, (void**)&p->d_partial, (size_t)p->cc_nsplit * p->cc_slot_stride * 8));
+    p->ccl = cc_launch_shape(p->cc, order, p->nfield, (int64_t)n3 / 32, p->sms);  // N^3 is a multiple of 32 for every N
+    PS_TRY(ps_alloc(p, (void**)&p->d_partial, (size_t)(p->ccl.rows() * p->ccl.stride()) * 8));
     PS_TRY(ps_alloc(p, (void**)&p->d_S, (size_t)std::max<int64_t>(1, p->nbins) * 8));
     PS_TRY(ps_alloc(p, (void**)&p->d_counts, (size_t)std::max<int64_t>(1, p->nbins) * 8));
     PS_TRY(ps_alloc(p, &p->d_in_stage, n3 * es));
@@ -677,19 +709,6 @@ static poly_status create_plan(PsPlan* p, int N, double L, int order, int nshell
     // exact counts (plan time, cached)
     PS_TRY(compute_counts(p, st));
     PS_CUDA(cudaMemcpy(p->d_counts, p->counts.data(), p->nbins * 8, cudaMemcpyHostToDevice));
-    if (ell > 0) {
-        // the counts used the plain tiles; the estimate's first leg reads the weighted fields
-        for (void* d : {p->d_cc_tiles, p->d_cc_field_ids, p->d_cc_rowf, p->d_cc_colf, p->d_cc_slot}) ps_free(p, d);
-        p->cc = CcTiles();
-        build_cc_tiles(p, p->cc, nshell);
-        PS_TRY(upload(p, &p->d_cc_tiles, p->cc.tiles));
-        PS_TRY(upload(p, &p->d_cc_field_ids, p->cc.field_ids));
-        PS_TRY(upload(p, &p->d_cc_rowf, p->cc.rowf));
-        PS_TRY(upload(p, &p->d_cc_colf, p->cc.colf));
-        PS_TRY(upload(p, &p->d_cc_slot, p->cc.slot));
-        if ((int64_t)p->cc.tiles.size() * kCcTM * kCcTN != p->cc_slot_stride)
-            return set_error(POLY_ERR_ARG, "multipole tiles differ in shape from the plain ones");
-    }
     PS_CUDA(cudaDeviceSynchronize());
     return POLY_OK;
 }
@@ -747,14 +766,11 @@ poly_status ps_fields(PsPlan* p, const void* delta, cudaStream_t st) {
 poly_status ps_sums(PsPlan* p, bool absval, cudaStream_t st) {
     cudaError_t e;
     if (p->prec == POLY_SPLIT_BF16 && !absval) return ps_tc_sums(p, st);
-    const size_t n3 = (size_t)p->N * p->N * p->N;
-    if ((e = ps_contract_cc(p->is_double, 0, absval ? 1 : 0, p->order >= 5 ? 3 : 2, p->d_fields, n3, p->nfield, (int64_t)n3, nullptr,
-                            (const PsTile*)p->d_cc_tiles, (int)p->cc.tiles.size(), (const int*)p->d_cc_field_ids,
-                            (const short4*)p->d_cc_rowf, (const short4*)p->d_cc_colf, p->cc_nsplit, p->cc_cps,
-                            p->d_partial, st)))
+    if ((e = ps_contract_cc(p->is_double, p->order, 0, absval ? 1 : 0, p->ccl, p->d_fields, nullptr,
+                            (const CcGroup*)p->d_cc_groups, (const CcTask*)p->d_cc_tasks, p->d_partial, st)))
         return cuda_error(e, "contraction");
     if (!absval) mark(p, 3, st);
-    if ((e = ps_reduce_slots(p->d_partial, p->cc_nsplit, p->cc_slot_stride, (const int64_t*)p->d_cc_slot, p->nbins,
+    if ((e = ps_reduce_slots(p->d_partial, (int)p->ccl.rows(), p->ccl.stride(), (const int64_t*)p->d_cc_slot, p->nbins,
                              p->d_S, st)))
         return cuda_error(e, "contraction");
     p->launches += 2;
@@ -994,20 +1010,45 @@ static int poly_diag_host_tables_impl(int N, int order, const double* edges, int
     PsPlan h;  // host tables only: no device call, no device memory
     std::vector<short> ln;
     PS_TRY(ps_plan_host_tables(&h, N, 1.0, order, nshell, edges, POLY_FP64, flags, ell, ln));
-    if (ell > 0) {  // as poly_plan_create_multipole leaves them: the first leg on the weighted slots
-        h.cc = CcTiles();
-        build_cc_tiles(&h, h.cc, nshell);
+    // every task as a tile: the runs of its legs are its local fields, a product of the first legs a row, of the
+    // rest a column
+    std::vector<int32_t> tl, fid;
+    std::vector<int16_t> rowf_, colf_;
+    std::vector<int64_t> tslot(h.cc.slot);
+    const int ra = cc_ra(order), cols = cc_span(order, true, ra, order), values = cc_span(order, true, 0, order);
+    for (const auto& first : h.cc.first) {
+        const int32_t row_off = (int32_t)rowf_.size() / 4, col_off = (int32_t)colf_.size() / 4, foff = (int32_t)fid.size();
+        std::array<int, 6> loc{};
+        for (int l = 0; l < order; l++) {
+            loc[l] = (int)fid.size() - foff;
+            for (int i = 0; i < cc_dim(order, true, l); i++) fid.push_back(std::min(first[l] + i, h.cc.nslot - 1));
+        }
+        auto records = [&](int l0, int l1, std::vector<int16_t>& out) {
+            const int cnt = cc_span(order, true, l0, l1);
+            for (int v = 0; v < cnt; v++) {
+                int16_t r[4] = {-1, -1, -1, -1};
+                for (int l = l1 - 1, w = v; l >= l0; l--) {
+                    r[l - l0] = (int16_t)(loc[l] + w % cc_dim(order, true, l));
+                    w /= cc_dim(order, true, l);
+                }
+                out.insert(out.end(), r, r + 4);
+            }
+            return cnt;
+        };
+        const int nrow = records(0, ra, rowf_), ncol = records(ra, order, colf_);
+        const int32_t rec[8] = {row_off, nrow, col_off, ncol, foff, (int32_t)fid.size() - foff, 1, 0};
+        tl.insert(tl.end(), rec, rec + 8);
     }
-    const int64_t n[7] = {h.nbins, (int64_t)h.cc.tiles.size(), (int64_t)h.cc.field_ids.size(),
-                          (int64_t)h.cc.rowf.size(), (int64_t)h.cc.colf.size(), (int64_t)ln.size() / 4,
-                          (int64_t)h.line_off.size()};
+    for (auto& v : tslot) v = v / values * 4096 + v % values / cols * 64 + v % cols;
+    const int64_t n[7] = {h.nbins, (int64_t)tl.size() / 8, (int64_t)fid.size(), (int64_t)rowf_.size() / 4,
+                          (int64_t)colf_.size() / 4, (int64_t)ln.size() / 4, (int64_t)h.line_off.size()};
     for (int i = 0; i < 7; i++) sizes[i] = n[i];
     if (bins) std::memcpy(bins, h.bins.data(), h.bins.size() * sizeof(int32_t));
-    if (tiles) std::memcpy(tiles, h.cc.tiles.data(), h.cc.tiles.size() * sizeof(PsTile));
-    if (field_ids) std::memcpy(field_ids, h.cc.field_ids.data(), h.cc.field_ids.size() * sizeof(int32_t));
-    if (rowf) std::memcpy(rowf, h.cc.rowf.data(), h.cc.rowf.size() * sizeof(short4));
-    if (colf) std::memcpy(colf, h.cc.colf.data(), h.cc.colf.size() * sizeof(short4));
-    if (slot) std::memcpy(slot, h.cc.slot.data(), h.cc.slot.size() * sizeof(int64_t));
+    if (tiles) std::memcpy(tiles, tl.data(), tl.size() * sizeof(int32_t));
+    if (field_ids) std::memcpy(field_ids, fid.data(), fid.size() * sizeof(int32_t));
+    if (rowf) std::memcpy(rowf, rowf_.data(), rowf_.size() * sizeof(int16_t));
+    if (colf) std::memcpy(colf, colf_.data(), colf_.size() * sizeof(int16_t));
+    if (slot) std::memcpy(slot, tslot.data(), tslot.size() * sizeof(int64_t));
     if (lines) std::memcpy(lines, ln.data(), ln.size() * sizeof(short));
     if (line_off) std::memcpy(line_off, h.line_off.data(), h.line_off.size() * sizeof(int32_t));
     return POLY_OK;
@@ -1219,8 +1260,7 @@ poly_status poly_plan_stats(poly_plan p, poly_stats* out) {
         const double n3 = (double)p->N * p->N * p->N;
         double f = 0;
         if (p->prec == POLY_SPLIT_BF16) f = ps_tc_executed_flops(p);
-        else
-            for (const auto& t : p->cc.tiles) f += 2.0 * 512.0 * __builtin_popcount(t.region_mask) * n3;
+        else f = 2.0 * (double)p->ccl.stride() * n3;
         out->contract_flops = f;
     }
     if (!p->ev_recorded) return POLY_OK;

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <array>
 #include <functional>
 #include <string>
 #include <vector>
@@ -9,11 +10,16 @@
 #include "../../include/polyspec.h"
 #include "kernels.h"
 
-struct CcTiles {
-    std::vector<PsTile> tiles;
-    std::vector<int> field_ids;
-    std::vector<short4> rowf, colf;  // up to three factors each (-1: none)
-    std::vector<int64_t> slot;  // per bin: tile * 64 * 64 + r * 64 + c
+// CUDA-core contraction tasks (host): each task's first field slot per leg, the blocks they are
+// grouped into and every bin's product.
+struct CcTasks {
+    std::vector<std::array<short, 6>> first;  // per task and leg: first field slot of its run
+    std::vector<CcTask> tasks;                // the same as offsets into their group's copy
+    std::vector<CcGroup> groups;
+    std::vector<int64_t> slot;                // per bin: task * values + product
+    int nslot = 0;                            // field slots the runs may name: [0, nslot)
+    int is_double = 0, max_used = 0;
+    int64_t ntask() const { return (int64_t)tasks.size(); }
 };
 
 // Largest number of shells a plan takes.  Host tables pack shell and field-slot
@@ -54,11 +60,9 @@ struct poly_plan_s {
     void* d_xpre = nullptr;    // x-pass output of the inverse transform
     size_t xpre_lines = 0;     // lines the x-pass buffer holds (indexed by global line offset)
     // CUDA-core contraction
-    CcTiles cc;
-    void *d_cc_tiles = nullptr, *d_cc_field_ids = nullptr, *d_cc_rowf = nullptr, *d_cc_colf = nullptr,
-         *d_cc_slot = nullptr;
-    int cc_nsplit = 1;
-    int64_t cc_cps = 0, cc_slot_stride = 0;
+    CcTasks cc;
+    CcLaunch ccl;
+    void *d_cc_tasks = nullptr, *d_cc_groups = nullptr, *d_cc_slot = nullptr;
     // workspace
     void* d_W = nullptr;       // forward intermediate, N x (2K+1)(K+1) complex
     void* d_fhat = nullptr;    // pruned half spectrum, (2K+1)(K+1)(2K+1) complex
@@ -101,7 +105,10 @@ void ps_set_last_error(const std::string& msg);
 // host-side tables (plan.cpp)
 void enumerate_bins(int nshell, const std::vector<double>& edges, int order, bool all_sorted, std::vector<int32_t>& out);
 void build_lines(const PsPlan* p, const double* e, int s, std::vector<short>& lines);
-void build_cc_tiles(PsPlan* p, CcTiles& t, int first_shift = 0);
+// tasks of the CUDA-core contraction for the plan's bins; first_shift > 0: the first leg reads slot k1 - 1 + first_shift
+void build_cc_tasks(const PsPlan* p, int is_double, int first_shift, CcTasks& t);
+// launch shape over nchunk 32-cell chunks of nf field slots; max_rows > 0 bounds the partial sums per task
+CcLaunch cc_launch_shape(const CcTasks& t, int order, int nf, int64_t nchunk, int sms, int64_t max_rows = 0);
 // the adjoint's entry tables (adjoint.cu); host only
 void ps_adj_entries(const PsPlan* p, std::vector<int>& moff, std::vector<short4>& ent, std::vector<int>& eoff,
                     std::vector<int>& ebins);
