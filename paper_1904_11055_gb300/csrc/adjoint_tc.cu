@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kAtThreads, 1)
                        const uint8_t* __restrict__ bhi_g, const uint8_t* __restrict__ blo_g, float* __restrict__ G,
                        int* __restrict__ err) {
     // every pointer below is smem_raw plus an offset, so that the compiler keeps shared-memory loads
-    extern __shared__ __align__(16) uint8_t smem_raw[];
+    extern __shared__ __align__(128) uint8_t smem_raw[];
     const int npairs = (ngroups + 1) / 2;
     const int pr = blockIdx.x % npairs, range = blockIdx.x / npairs;
     AtGroup gm[2];
@@ -286,6 +286,367 @@ __global__ void __launch_bounds__(kAtThreads, 1)
     if (tid == 0 && *s_abort) atomicExch(err, tc::kErrTimeout);
 }
 
+// ---------------------------------------------------------------------------------
+// The same gradient as one GEMM over pairs of shells, for up to 64 shells:
+//   G_m(x) = sum_p P_p(x) W[p][m],  P_p = D_i D_j of the pair p = (i <= j).
+// M = 128 cells (TMEM lanes), K = the pairs, N = the shells m.  The products are formed in FP32, split into
+// bf16 hi + lo and written to TMEM (A); the weights (B, hi and lo) stream through shared memory.
+//
+// Why: T[x][(m, j)] = sum_i W_m[i][j] D_i (above) multiplies every cell with 3,584 columns x 64 shells and
+// reduces the columns on the CUDA cores; the pairs need 2,304 products a cell, 64 columns, no reduction, and
+// skip the columns that a pair's triangles do not reach (at 64 shells a quarter of them).  256^3 / 64 shells:
+// 26.2 -> 13.9 ms (10.4 without what the precision asks for, below).  What bounds it: the producers' instructions
+// (seven per two products and as many around them) and the barriers of each chunk; without the lo x lo products
+// 62 % of the issue slots, the ALU pipe of the bf16 conversions 48 % busy, the tensor pipe 37 %.
+//
+// K comes in chunks of 64 pairs: 8 consecutive i by 8 consecutive j, so that a lane keeps its 8 D_j in
+// registers over a run of chunks and loads 8 values per 64 products.  (Chunks of 32 pairs ran 12.6 ms instead of
+// 10.4 at 256^3 / 64 shells, 10 ms of it without the products and two thirds of the MMAs: the barriers around a
+// chunk set the pace.)  A chunk's columns are the 16-column blocks that hold one of its weights (the first chunk
+// of a segment takes them all and overwrites, which starts the sums).  The weights of absent entries are zero.
+//
+// A block takes tiles of 256 cells (two M tiles).  12 producer warps in three groups: group g forms both M
+// tiles' products of chunks g, g + 3, ... (chunk c in A slot c mod 3; one cell of each tile a lane, so that a
+// chunk's barriers and addresses serve 128 products a lane), warp % 4 is the lane quadrant.  One issuer warp per
+// M tile, one warp for the copies: the tile's fields (one bulk copy, two buffers) and the chunks' weights (a
+// ring).  The accumulators are summed over segments of a few chunks only, because the tensor core's FP32
+// accumulation truncates (relative 2^-25 per MMA): the producer warps add a finished segment to their FP32 sums
+// (rounded to nearest).  The lo x lo products are added too (the tensor pipe has the room), and up to 32 shells
+// the cross products have sums of their own, so that fewer additions truncate the large ones: the error against
+// 64 bits is then no larger than that of the columns (m, j).
+constexpr int kAqCells = 256;    // cells of a tile
+constexpr int kAqMaxShells = 64;
+constexpr int kAqProd = 12;      // producer warps
+constexpr int kAqThreads = 32 * (kAqProd + 3);
+constexpr int kAqGroups = 3;     // groups of four producer warps
+constexpr int kAqSlots = 3;      // A slots (>= kAqGroups), each both M tiles' products of one chunk
+constexpr int kAqRing = 4;       // chunks of weights in shared memory
+// chunks per accumulation segment (16 accumulations each; 3 at 33-48 shells), above 32 shells: 256^3 / 64 shells
+// 20.7 ms a gradient with 6 (error 3.4e-6 against 64 bits), 21.1 with 5 (3.2e-6), 21.6 with 4 (3.1e-6)
+constexpr int kAqSeg = 4;
+constexpr int kAqSegSplit = 12;  // with the cross products in sums of their own (48), up to 32 shells
+constexpr int kAqDelay = kAqGroups;      // chunks after a segment's end at which a group reads its sums: one chunk of each group
+constexpr int kAqBar = 64;       // mbarriers and flags, in 8-byte words
+
+struct AqChunk {
+    int jb, i0;      // first j, first i (8 of each); jb < 0: no products (nn = 0)
+    int n0, nn;      // columns [n0, n0 + nn)
+    int b_off;       // byte offset of its weights (hi, then lo: nn * 128 bytes each)
+    int first, last; // first / last chunk of its segment
+    int end;         // entry s: last chunk of the tile's segment s
+};
+
+// weights to their places: hi at place, lo lo_off bytes after it
+__global__ void aq_scatter_kernel(const float* __restrict__ w, const int2* __restrict__ place, int nent,
+                                  uint8_t* __restrict__ b) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nent; e += gridDim.x * blockDim.x) {
+        const int2 p = place[e];
+        const float v = w[e];
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
+        *reinterpret_cast<uint16_t*>(b + p.x) = *reinterpret_cast<const uint16_t*>(&h);
+        *reinterpret_cast<uint16_t*>(b + p.x + p.y) = *reinterpret_cast<const uint16_t*>(&l);
+    }
+}
+
+__global__ void __launch_bounds__(kAqThreads, 1)
+    at_pairs_kernel(const float* __restrict__ D, int nshell, int64_t ncell, int ntile, const AqChunk* __restrict__ chunks,
+                    int nchunk, int nblk16, const uint8_t* __restrict__ b_g, int b_stage, float* __restrict__ G,
+                    int* __restrict__ err) {
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    const int row = 128, qbytes = nshell * row, tile_bytes = 8 * qbytes;  // [8 chunks of 32 cells][nshell][32]
+    uint8_t* s_d = smem_raw;                         // two tiles
+    uint8_t* s_b = s_d + 2 * (size_t)tile_bytes;     // kAqRing x b_stage
+    AqChunk* s_ch = reinterpret_cast<AqChunk*>(s_b + (size_t)kAqRing * b_stage);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(s_ch + nchunk);
+    uint64_t* d_full = bars;              // [2]
+    uint64_t* d_free = bars + 2;          // [2] every producer warp is done with the tile
+    uint64_t* b_full = bars + 4;          // [kAqRing]
+    uint64_t* b_free = bars + 12;         // [kAqRing] both M tiles' MMAs have read the chunk
+    uint64_t* produced = bars + 20;       // [kAqSlots]
+    uint64_t* freed = bars + 28;          // [kAqSlots] both M tiles' MMAs have read the slot
+    uint64_t* acc_full = bars + 36;       // a segment's MMAs are complete, both M tiles'
+    uint64_t* acc_free = bars + 37;       // its sums have been read
+    uint64_t* drain = bars + 38;          // [2]
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 40);
+    volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < nchunk * (int)(sizeof(AqChunk) / 4); i += kAqThreads)
+        reinterpret_cast<int*>(s_ch)[i] = reinterpret_cast<const int*>(chunks)[i];
+    if (tid == 0) {
+        for (int b = 0; b < 2; b++) {
+            tc::mbar_init(d_full + b, 1);
+            tc::mbar_init(d_free + b, kAqProd);
+            tc::mbar_init(drain + b, 1);
+        }
+        for (int b = 0; b < kAqRing; b++) {
+            tc::mbar_init(b_full + b, 1);
+            tc::mbar_init(b_free + b, 2);
+        }
+        for (int b = 0; b < kAqSlots; b++) {
+            tc::mbar_init(produced + b, 4);
+            tc::mbar_init(freed + b, 2);
+        }
+        tc::mbar_init(acc_full, 2);
+        tc::mbar_init(acc_free, kAqProd);
+        tc::mbar_fence_init();
+        *s_abort = 0;
+    }
+    if (warp == kAqProd) {
+        tc::tmem_alloc(s_tmem, 512);
+        tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *s_tmem;
+    // accumulators of M tile t at column 64 t, up to 32 shells the cross products' 32 columns on; A slot s of M tile t at 128 + 128 s + 64 t
+    const int ntl = ((int)blockIdx.x < ntile) ? (ntile - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const uint32_t cross = nblk16 <= 2 ? 32u : 0u;
+    const int total = ntl * nchunk;  // chunks this block runs (a tile's chunks in a row, tile after tile)
+
+    if (warp == kAqProd + 2) {
+        // ------------------------------------------------------------ copies
+        if (tc::elect_one()) {
+            int d_iss = 0, b_iss = 0;
+            bool ok = true;
+            auto load_tile = [&](int k) {
+                tc::mbar_arrive_expect_tx(d_full + (k & 1), (uint32_t)tile_bytes);
+                tc::bulk_load(s_d + (size_t)(k & 1) * tile_bytes,
+                              D + ((size_t)blockIdx.x + (size_t)k * gridDim.x) * kAqCells * nshell, (uint32_t)tile_bytes,
+                              d_full + (k & 1));
+                d_iss = k + 1;
+            };
+            if (ntl > 0) load_tile(0);
+            const int at = nchunk - 1 < 8 ? nchunk - 1 : 8;  // the next tile's fields a few chunks into a tile
+            int rs = 0, c = 0, k = 0;
+            uint32_t rph = 1;
+            for (int cg = 0; cg < total && ok; cg++) {
+                if (c == at && k + 1 < ntl) {
+                    if (k >= 1) ok = tc::mbar_wait(d_free + ((k + 1) & 1), (uint32_t)(((k - 1) >> 1) & 1), s_abort);
+                    if (!ok) break;
+                    load_tile(k + 1);
+                }
+                if (cg >= kAqRing && !tc::mbar_wait(b_free + rs, rph, s_abort)) break;
+                const AqChunk ch = s_ch[c];
+                tc::mbar_arrive_expect_tx(b_full + rs, (uint32_t)(ch.nn * 256));
+                if (ch.nn > 0)
+                    tc::bulk_load(s_b + (size_t)rs * b_stage, b_g + ch.b_off, (uint32_t)(ch.nn * 256), b_full + rs);
+                b_iss = cg + 1;
+                if (++rs == kAqRing) {
+                    rs = 0;
+                    rph ^= 1u;
+                }
+                if (++c == nchunk) {
+                    c = 0;
+                    k++;
+                }
+            }
+            // every copy started lands before the block exits
+            volatile int no_abort = 0;
+            for (int q = d_iss > 2 ? d_iss - 2 : 0; q < d_iss; q++)
+                tc::mbar_wait(d_full + (q & 1), (uint32_t)((q >> 1) & 1), &no_abort);
+            for (int q = b_iss > kAqRing ? b_iss - kAqRing : 0; q < b_iss; q++)
+                tc::mbar_wait(b_full + q % kAqRing, (uint32_t)((q / kAqRing) & 1), &no_abort);
+        }
+        __syncwarp();
+    } else if (warp >= kAqProd) {
+        // ------------------------------------------------------------ MMA issue for M tile t
+        const int t = warp - kAqProd;
+        const bool el = tc::elect_one();
+        // K-major core matrices of 8 rows x 16 bytes: 128 bytes along K, 1024 bytes per 8 columns
+        const uint64_t desc_k = ((uint64_t)((1024u >> 4) | (1u << 14)) << 32) | (uint64_t)((128u >> 4) << 16);
+        int rs = 0, c = 0, gs = 0;
+        uint32_t rph = 0;
+        for (int cg = 0; cg < total; cg++) {
+            const AqChunk ch = s_ch[c];
+            const int slot = cg % kAqSlots;
+            if (ch.first && gs >= 1 && !tc::mbar_wait_warp(acc_free, (uint32_t)((gs - 1) & 1), s_abort))
+                break;
+            if (!tc::mbar_wait_warp(b_full + rs, rph, s_abort)) break;
+            if (!tc::mbar_wait_warp(produced + slot, (uint32_t)((cg / kAqSlots) & 1), s_abort)) break;
+            tc::fence_after_sync();
+            if (el) {
+                const uint32_t d = tmem + (uint32_t)(64 * t + ch.n0);
+                const uint32_t a = tmem + 128u + (uint32_t)(128 * slot + 64 * t);
+                const uint32_t bh = tc::smem_u32(s_b + (size_t)rs * b_stage), bl = bh + (uint32_t)(ch.nn * 128);
+                const uint32_t idesc = tc::idesc_bf16(128, ch.nn);
+                const uint32_t dx = d + cross, fx = ch.first && cross ? 0u : 1u;
+#pragma unroll
+                for (int ks = 0; ks < 4 && ch.nn > 0; ks++) {
+                    const uint64_t dh = desc_k | (uint64_t)(((bh + ks * 256) >> 4) & 0x3FFFu);
+                    const uint64_t dl = desc_k | (uint64_t)(((bl + ks * 256) >> 4) & 0x3FFFu);
+                    const uint32_t ah = a + (uint32_t)(8 * ks), al = ah + 32u;
+                    tc::mma_ts(d, ah, dh, idesc, ks == 0 && ch.first ? 0u : 1u);  // hi x hi
+                    tc::mma_ts(dx, ah, dl, idesc, ks == 0 ? fx : 1u);             // hi x lo
+                    tc::mma_ts(dx, al, dh, idesc, 1u);                            // lo x hi
+                    tc::mma_ts(dx, al, dl, idesc, 1u);                            // lo x lo
+                }
+                tc::mma_commit(freed + slot);
+                tc::mma_commit(b_free + rs);
+                if (ch.last) tc::mma_commit(acc_full);
+            }
+            __syncwarp();
+            gs += ch.last;
+            if (++rs == kAqRing) {
+                rs = 0;
+                rph ^= 1u;
+            }
+            if (++c == nchunk) c = 0;
+        }
+        // every MMA started completes before the columns are freed
+        if (el) {
+            tc::mma_commit(drain + t);
+            volatile int no_abort = 0;
+            tc::mbar_wait(drain + t, 0, &no_abort);
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------------ products, sums
+        const int q = warp & 3, g = warp >> 2;  // lane quadrant; group: chunks g, g + 3, ...
+        const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+        const uint32_t d0 = tc::smem_u32(s_d) + (uint32_t)(q * qbytes + lane * 4);  // M tile 0's cell; tile 1's is 4 chunks on
+        const uint32_t a0 = tmem + lane_base + 128u;
+        // sums of this lane's cells: items g, g + 3, g + 6 of the (16-column block, M tile) pairs 2 b + t
+        float sums[3][16];
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = 0; j < 16; j++) sums[i][j] = 0.f;
+        int gs = 0, ss = 0, sk = 0;  // segments added so far; the next one's number within its tile, and the tile
+        int seg_end = ntl > 0 ? s_ch[0].end : 0;  // its last chunk
+        auto add_segment = [&]() -> bool {
+            if (!tc::mbar_wait_warp(acc_full, (uint32_t)(gs & 1), s_abort)) return false;
+            tc::fence_after_sync();
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                const int item = g + 3 * i;
+                if (item < 2 * nblk16) {
+                    uint32_t v[16];
+                    tc::tmem_ld16(tmem + lane_base + (uint32_t)(64 * (item & 1) + 16 * (item >> 1)), v);
+                    tc::tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 16; j++) sums[i][j] += __uint_as_float(v[j]);
+                    if (cross) {
+                        tc::tmem_ld16(tmem + lane_base + (uint32_t)(64 * (item & 1) + 16 * (item >> 1)) + cross, v);
+                        tc::tmem_ld_wait();
+#pragma unroll
+                        for (int j = 0; j < 16; j++) sums[i][j] += __uint_as_float(v[j]);
+                    }
+                }
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(acc_free);
+            gs++;
+            if (s_ch[ss].end + 1 == nchunk) {  // the tile's last segment
+                const int64_t cell0 = ((int64_t)blockIdx.x + (int64_t)sk * gridDim.x) * kAqCells + 32 * q + lane;
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                    const int item = g + 3 * i, m0 = 16 * (item >> 1);
+                    float* out = G + (size_t)m0 * ncell + cell0 + 128 * (item & 1);
+#pragma unroll
+                    for (int j = 0; j < 16; j++) {
+                        if (m0 + j < nshell) out[0] = sums[i][j];
+                        out += ncell;
+                        sums[i][j] = 0.f;
+                    }
+                }
+                ss = -1;
+                sk++;
+            }
+            ss++;
+            seg_end = sk < ntl ? sk * nchunk + s_ch[ss].end : total + kAqDelay;  // none left: never reached
+            return true;
+        };
+        uint64_t dj[2][4];  // D_j in pairs, both cells
+        int jb_of = -1;
+        bool ok = true;
+        int c = g, k = 0, k_have = -1;  // chunk of the tile, tile; tile whose fields this warp has waited for
+        int slot = g;                   // cg mod kAqSlots
+        uint32_t ph = 1;                // phase of freed[] that releases the slot
+        for (int cg = g; cg < total; cg += kAqGroups, c += kAqGroups) {
+            while (c >= nchunk) {
+                c -= nchunk;
+                k++;
+            }
+            while (ok && seg_end + kAqDelay <= cg) ok = add_segment();
+            if (!ok) break;
+            while (k_have < k) {  // leave the tiles before, wait for the fields of tile k
+                if (k_have >= 0 && lane == 0) tc::mbar_arrive(d_free + (k_have & 1));
+                k_have++;
+                jb_of = -1;
+                if (!(ok = tc::mbar_wait_warp(d_full + (k_have & 1), (uint32_t)((k_have >> 1) & 1), s_abort))) break;
+            }
+            if (!ok) break;
+            const int2 ch = *reinterpret_cast<const int2*>(s_ch + c);  // first j, first i
+            const uint32_t db = d0 + (uint32_t)((k & 1) * tile_bytes);
+            auto ld = [&](uint32_t a) {
+                float v;
+                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+                return v;
+            };
+            const bool some = ch.x >= 0;
+            if (some && ch.x != jb_of) {  // shells past the last read the last one's field; their weights are zero
+                jb_of = ch.x;
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const uint32_t r0 = db + (uint32_t)(min(ch.x + 2 * j, nshell - 1) * row);
+                    const uint32_t r1 = db + (uint32_t)(min(ch.x + 2 * j + 1, nshell - 1) * row);
+#pragma unroll
+                    for (int t = 0; t < 2; t++) dj[t][j] = tc::pack2(ld(r0 + t * 4 * qbytes), ld(r1 + t * 4 * qbytes));
+                }
+            }
+            if (cg >= kAqSlots && !tc::mbar_wait_warp(freed + slot, ph, s_abort)) {
+                ok = false;
+                break;
+            }
+            tc::fence_after_sync();
+            const uint32_t as = a0 + (uint32_t)(128 * slot);
+            // K order: i0's 8 pairs, i0 + 1's, ...: two per column; hi in columns 0-31, lo in 32-63
+            const bool whole = ch.y + 7 < nshell;
+#pragma unroll
+            for (int t = 0; t < 2; t++) {
+#pragma unroll
+                for (int i = 0; i < 8 && some; i += 4) {
+                    uint32_t hi[16], lo[16];
+                    float di[4];
+                    const uint32_t r = db + (uint32_t)((ch.y + i) * row + t * 4 * qbytes);
+#pragma unroll
+                    for (int u = 0; u < 4; u++)
+                        di[u] = ld(whole ? r + u * row : db + (uint32_t)(min(ch.y + i + u, nshell - 1) * row + t * 4 * qbytes));
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        const uint64_t d2 = tc::pack2(di[u], di[u]);
+#pragma unroll
+                        for (int j = 0; j < 4; j++) tc::split_pair(tc::mul2(d2, dj[t][j]), hi[4 * u + j], lo[4 * u + j]);
+                    }
+                    tc::tmem_st16(as + (uint32_t)(64 * t + 4 * i), hi);
+                    tc::tmem_st16(as + (uint32_t)(64 * t + 32 + 4 * i), lo);
+                }
+            }
+            tc::tmem_st_wait();
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(produced + slot);
+            slot += kAqGroups;
+            if (slot >= kAqSlots) {
+                slot -= kAqSlots;
+                ph ^= 1u;
+            }
+        }
+        while (ok && sk < ntl) ok = add_segment();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == kAqProd) {
+        tc::fence_after_sync();
+        tc::tmem_dealloc(tmem, 512);
+    }
+    if (tid == 0 && *s_abort) atomicExch(err, tc::kErrTimeout);
+}
+
 }  // namespace ps
 
 using namespace ps;
@@ -298,6 +659,12 @@ struct AtState {
     void *d_groups = nullptr, *d_chunks = nullptr, *d_pos = nullptr, *d_bhi = nullptr, *d_blo = nullptr;
     int* d_err = nullptr;
     int nent = 0;
+    // the pair form (up to kAqMaxShells shells)
+    bool pairs = false;
+    std::vector<AqChunk> chunks;
+    std::vector<int2> place;
+    int nblk16 = 0;
+    void* d_b = nullptr;
 };
 
 // shared memory of a block whose pair of groups has nc0 and nc1 chunks
@@ -386,6 +753,64 @@ static poly_status at_build_tables(const PsPlan* p, const std::vector<int>& ent_
     return POLY_OK;
 }
 
+// Host tables of the pair form: the chunks of 8 i by 8 j that hold an entry, their columns, segments and B
+// offsets, and the B place of every entry (and the offset of its lo part).  Touches no device.
+static void aq_build_tables(const PsPlan* p, const std::vector<int>& ent_m, const std::vector<short4>& ent, AtState* S,
+                            size_t& b_total) {
+    std::map<std::pair<int, int>, std::pair<int, int>> cols;  // (j / 8, i / 8) -> first and last 16-column block
+    for (size_t e = 0; e < ent.size(); e++) {
+        const std::pair<int, int> key{ent[e].y / 8, ent[e].x / 8};
+        const int b = ent_m[e] / 16;
+        auto r = cols.insert({key, {b, b}});
+        r.first->second.first = std::min(r.first->second.first, b);
+        r.first->second.second = std::max(r.first->second.second, b);
+    }
+    if (cols.empty()) cols[{0, 0}] = {0, 0};  // no entry at all: one chunk of zeros
+    S->nblk16 = (p->nshell + 15) / 16;
+    // every group takes part in every tile (it is what frees the tile's fields): at least kAqGroups chunks, the
+    // added ones without products
+    const int n = std::max<int>((int)cols.size(), kAqGroups), per = S->nblk16 <= 2 ? kAqSegSplit : S->nblk16 == 3 ? kAqSeg - 1 : kAqSeg;
+    const int nseg = (n + per - 1) / per;
+    std::map<std::pair<int, int>, int> at;
+    b_total = 0;
+    int k = 0, seg = 0;
+    for (auto& kv : cols) {  // j blocks ascending, i ascending within
+        AqChunk c{};
+        c.jb = 8 * kv.first.first;
+        c.i0 = 8 * kv.first.second;
+        c.first = k == n * seg / nseg;
+        c.last = k + 1 == n * (seg + 1) / nseg;
+        c.n0 = c.first ? 0 : 16 * kv.second.first;
+        c.nn = c.first ? 16 * S->nblk16 : 16 * (kv.second.second + 1 - kv.second.first);
+        c.b_off = (int)b_total;
+        b_total += (size_t)c.nn * 256;
+        at[kv.first] = k++;
+        seg += c.last;
+        S->chunks.push_back(c);
+    }
+    for (; k < n; k++) {
+        AqChunk c{};
+        c.jb = -1;
+        c.first = k == n * seg / nseg;
+        c.last = k + 1 == n * (seg + 1) / nseg;
+        seg += c.last;
+        S->chunks.push_back(c);
+    }
+    for (int t = 0; t < nseg; t++) S->chunks[t].end = n * (t + 1) / nseg - 1;
+    S->place.resize(ent.size());
+    for (size_t e = 0; e < ent.size(); e++) {
+        const AqChunk& c = S->chunks[at.at({ent[e].y / 8, ent[e].x / 8})];
+        const int kk = (ent[e].x - c.i0) * 8 + ent[e].y - c.jb, nc = ent_m[e] - c.n0;
+        S->place[e] = make_int2(c.b_off + nc / 8 * 1024 + kk / 8 * 128 + nc % 8 * 16 + kk % 8 * 2, c.nn * 128);
+    }
+    S->nent = (int)ent.size();
+    // at least half the SM's shared memory: one block per SM, so no block waits in tcgen05.alloc for another
+    S->smem = std::max<size_t>(2 * (size_t)kAqCells * p->nshell * 4 + (size_t)kAqRing * S->nblk16 * 16 * 256 +
+                                   S->chunks.size() * sizeof(AqChunk) + kAqBar * 8,
+                               116 * 1024);
+    S->pairs = true;
+}
+
 poly_status ps_at_prepare(PsPlan* p, const std::vector<int>& ent_m, const std::vector<short4>& ent, AtState** out) {
     *out = nullptr;
     const int64_t ncell = (int64_t)p->N * p->N * p->N;
@@ -394,7 +819,12 @@ poly_status ps_at_prepare(PsPlan* p, const std::vector<int>& ent_m, const std::v
     if (!S) return POLY_ERR_ALLOC;
     std::vector<int> chunks, pos;
     size_t b_total = 0;
-    if (poly_status s0 = at_build_tables(p, ent_m, ent, S, chunks, pos, b_total)) {
+    // Pairs up to 64 shells (two M tiles' sums and three A slots fill tensor memory), columns (m, j) beyond; and
+    // for up to four shells on large grids, where a tile's single chunk leaves the pairs' barriers bare (256^3 / 3
+    // shells: gradient 1.16 against 1.10 ms; 5 shells 1.26 against 1.31, 160^3 / 4 shells 0.47 against 0.50).
+    if (p->nshell <= kAqMaxShells && !(p->nshell <= 4 && ncell > (int64_t)160 * 160 * 160)) {
+        aq_build_tables(p, ent_m, ent, S, b_total);
+    } else if (poly_status s0 = at_build_tables(p, ent_m, ent, S, chunks, pos, b_total)) {
         delete S;
         return s0;
     }
@@ -404,6 +834,20 @@ poly_status ps_at_prepare(PsPlan* p, const std::vector<int>& ent_m, const std::v
         return cudaMemcpy(*d, h, bytes, cudaMemcpyHostToDevice) ? POLY_ERR_CUDA : POLY_OK;
     };
     poly_status s;
+    if (S->pairs) {
+        if ((s = up(&S->d_chunks, S->chunks.data(), S->chunks.size() * sizeof(AqChunk))) ||
+            (s = up(&S->d_pos, S->place.data(), std::max<size_t>(1, S->place.size()) * sizeof(int2))) ||
+            (s = ps_alloc(p, &S->d_b, b_total)) || (s = ps_alloc(p, (void**)&S->d_err, 16))) {
+            delete S;
+            return s;
+        }
+        if (cudaMemset(S->d_b, 0, b_total) || cudaMemset(S->d_err, 0, 16)) {
+            delete S;
+            return POLY_ERR_CUDA;
+        }
+        *out = S;
+        return POLY_OK;
+    }
     if ((s = up(&S->d_groups, S->groups.data(), S->groups.size() * sizeof(AtGroup))) ||
         (s = up(&S->d_chunks, chunks.data(), chunks.size() * 4)) ||
         (s = up(&S->d_pos, pos.data(), std::max<size_t>(1, pos.size()) * 4)) ||
@@ -483,6 +927,18 @@ extern "C" int poly_diag_adj_tables(int N, int order, const double* edges, int n
 // G[m][x] for all m from the plan's fields and the entry weights w (FP32, entry order).
 cudaError_t ps_at_contract(PsPlan* p, AtState* S, const float* w, cudaStream_t st) {
     const int nb = std::max(1, std::min(1024, (S->nent + 255) / 256));
+    if (S->pairs) {
+        aq_scatter_kernel<<<nb, 256, 0, st>>>(w, (const int2*)S->d_pos, S->nent, (uint8_t*)S->d_b);
+        cudaError_t e = cudaGetLastError();
+        if (e) return e;
+        if ((e = cudaFuncSetAttribute(at_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S->smem))) return e;
+        const int64_t ncell = (int64_t)p->N * p->N * p->N;
+        const int ntile = (int)(ncell / kAqCells);  // N^3 is a multiple of 256
+        at_pairs_kernel<<<std::min(p->sms, ntile), kAqThreads, S->smem, st>>>(
+            (const float*)p->d_fields, p->nshell, ncell, ntile, (const AqChunk*)S->d_chunks, (int)S->chunks.size(), S->nblk16,
+            (const uint8_t*)S->d_b, S->nblk16 * 16 * 256, (float*)p->d_G, S->d_err);
+        return cudaGetLastError();
+    }
     at_scatter_kernel<<<nb, 256, 0, st>>>(w, (const int*)S->d_pos, S->nent, (uint16_t*)S->d_bhi, (uint16_t*)S->d_blo);
     cudaError_t e = cudaGetLastError();
     if (e) return e;

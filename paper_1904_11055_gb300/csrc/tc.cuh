@@ -233,6 +233,42 @@ PS_DEV void split2_prod_x2(float x0, float y0, float x1, float y1, uint32_t& hi,
         : "f"(x0), "f"(x1), "f"(y0), "f"(y1));
 }
 
+// Pairs of FP32 values as one 64-bit value (x in the low half): they stay in an aligned register pair, where a
+// packed operation on two separate floats costs moves to build it.
+PS_DEV uint64_t pack2(float x, float y) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    return v;
+}
+PS_DEV uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+PS_DEV void lds2x2(uint32_t a, uint64_t& x, uint64_t& y) {  // 16 bytes of shared memory: two pairs
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "r"(a));
+}
+// hi = RN_bf16 pair of v; lo = RN_bf16 pair of the residuals v - hi, taken with one packed FP32
+// subtraction (exact: hi is within a factor 2 of each value).
+PS_DEV void split_pair(uint64_t v, uint32_t& hi, uint32_t& lo) {
+    asm("{\n\t"
+        ".reg .b64 ha, ra;\n\t"
+        ".reg .b32 h, h0, h1;\n\t"
+        ".reg .f32 p0, p1, r0, r1;\n\t"
+        "mov.b64 {p0, p1}, %2;\n\t"
+        "cvt.rn.bf16x2.f32 h, p1, p0;\n\t"
+        "shl.b32 h0, h, 16;\n\t"
+        "and.b32 h1, h, 0xffff0000;\n\t"
+        "mov.b64 ha, {h0, h1};\n\t"
+        "sub.rn.f32x2 ra, %2, ha;\n\t"
+        "mov.b64 {r0, r1}, ra;\n\t"
+        "cvt.rn.bf16x2.f32 %1, r1, r0;\n\t"
+        "mov.b32 %0, h;\n\t"
+        "}"
+        : "=r"(hi), "=r"(lo)
+        : "l"(v));
+}
+
 // hi = RN_bf16 pair of (a, b); lo = RN_bf16 pair of the residuals (a, b) - hi, taken
 // with one packed FP32 subtraction (exact: hi is within a factor 2 of each value).
 PS_DEV void split2_fast(float a, float b, uint32_t& hi, uint32_t& lo) {

@@ -1,6 +1,8 @@
 """The CUDA-core adjoint's blocks of output shells (eight in FP32, four in FP64) at their edges, against the FP64 oracle's gradient:
 one shell, a partial block, exactly one block or two, one shell more, and several blocks, in every order it serves
-(orders 2 and 4 of split-BF16 plans run here too)."""
+(orders 2 and 4 of split-BF16 plans run here too).  And the tensor-core adjoint's chunks of 8 by 8 shells and
+16-column blocks: partial ones, one chunk, an odd and an even count of them, several accumulation segments, the
+most shells of the pair form, and one more (narrow shells, some of them empty), which takes the other form."""
 import numpy as np
 import pytest
 
@@ -15,20 +17,29 @@ pytestmark = pytest.mark.gpu
 TOL = {"fp32": 2e-5, "split_bf16": 2e-5, "fp64": 1e-10}  # of the largest component, as the other adjoint tests
 
 
-@pytest.mark.parametrize("N,order,nshell,prec,flags", [
-    (16, 3, 1, "fp32", 0), (32, 3, 7, "fp32", 0), (32, 3, 8, "fp64", 0), (32, 3, 9, "fp32", 0), (64, 3, 19, "fp32", 0),
-    (32, 2, 11, "fp32", ps.POLY_BINS_ALL_SORTED), (24, 2, 8, "fp64", 0), (32, 4, 7, "fp32", 0), (24, 4, 5, "split_bf16", 0),
-    (48, 4, 9, "fp64", 0), (32, 3, 9, "fp64", ps.POLY_BINS_ALL_SORTED)])
-def test_gradient_blocks_match_oracle(N, order, nshell, prec, flags):
-    e = fieldgen.unit_edges(nshell)
-    d = fieldgen.field("lognormal", N, 70 + nshell, np.float32)
-    plan = ps.Plan(N, 500.0, order, e, prec, flags)
-    w = np.random.default_rng(nshell).standard_normal(plan.nbins) * (plan.counts > 0)
+def check(N, order, edges, prec, flags, seed):
+    d = fieldgen.field("lognormal", N, seed, np.float32)
+    plan = ps.Plan(N, 500.0, order, edges, prec, flags)
+    w = np.random.default_rng(seed).standard_normal(plan.nbins) * (plan.counts > 0)
     x = torch.from_numpy(d).cuda().to(plan.real_dtype)
     for _ in range(2):  # a second call finds the first one's weights and tables
         g = plan.backward(x, torch.from_numpy(w).cuda())
     plan.sync()
     some = plan.counts > 0
-    ref = oracle.gradient(d.astype(np.float64), 500.0, e, order, plan.bins[some], plan.counts[some], w[some])
+    ref = oracle.gradient(d.astype(np.float64), 500.0, edges, order, plan.bins[some], plan.counts[some], w[some])
     assert np.abs(g.double().cpu().numpy() - ref).max() <= TOL[prec] * np.abs(ref).max()
     plan.close()
+
+
+@pytest.mark.parametrize("N,nshell,width", [(16, 1, 1.0), (16, 4, 1.0), (32, 5, 1.0), (32, 9, 1.0), (48, 13, 1.0), (64, 16, 1.0),
+                                            (64, 17, 1.0), (32, 33, 0.3), (32, 64, 0.15), (32, 65, 0.15)])
+def test_pair_gradient_matches_oracle(N, nshell, width):
+    check(N, 3, fieldgen.unit_edges(nshell, width), "split_bf16", 0, 170 + nshell)
+
+
+@pytest.mark.parametrize("N,order,nshell,prec,flags", [
+    (16, 3, 1, "fp32", 0), (32, 3, 7, "fp32", 0), (32, 3, 8, "fp64", 0), (32, 3, 9, "fp32", 0), (64, 3, 19, "fp32", 0),
+    (32, 2, 11, "fp32", ps.POLY_BINS_ALL_SORTED), (24, 2, 8, "fp64", 0), (32, 4, 7, "fp32", 0), (24, 4, 5, "split_bf16", 0),
+    (48, 4, 9, "fp64", 0), (32, 3, 9, "fp64", ps.POLY_BINS_ALL_SORTED)])
+def test_gradient_blocks_match_oracle(N, order, nshell, prec, flags):
+    check(N, order, fieldgen.unit_edges(nshell), prec, flags, 70 + nshell)
