@@ -467,6 +467,9 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
             // drain the accumulators after the last chunk of a window
             win.advance_to(i, window);
             if (i == win.end || i == nch - 1) {
+                // the window before must be over first: this team may not have drained it, and after a last window
+                // of fewer chunks than slots its MMAs can still be running, when the parity below would pass early
+                if (win.index > 0 && !tc::mbar_wait_warp(acc_ready, (uint32_t)((win.index - 1) & 1), s_abort)) break;
                 if (!tc::mbar_wait_warp(acc_ready, (uint32_t)(win.index & 1), s_abort)) break;
                 tc::fence_after_sync();
                 for (int g = half; g < acc_cols / 16; g += 2) {
