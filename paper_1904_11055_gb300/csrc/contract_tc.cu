@@ -420,6 +420,12 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
         TcWindow win(team, window);
         for (int i = team < nteams ? team : nch; i < nch; i += nteams) {
             if (!tc::mbar_wait_warp(&full[st], ph_full, s_abort)) break;
+            const uint32_t D = sd0 + (uint32_t)(st * stage_bytes);
+            // two teams: the first tile's products before the wait for the slot, which they then cover (two
+            // teams, three slots: trispectrum 256^3 / 32 shells 12.95 -> 12.66 ms; three teams cover each other's
+            // waits and have no registers for it)
+            uint32_t v0[16];
+            if (TEAMS == 2) tc_row_products<RA>(D + key1[0], D + key2[0], RA == 3 ? D + key3[0] : 0u, v0);
             const int slot = i % nslots, use = i / nslots;  // slot and its use count
             if (use > 0) {
                 // the MMAs of chunk i - nslots have read the slot
@@ -429,16 +435,19 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
             const uint32_t Bh = Bbase + (uint32_t)(2 * slot * bbuf_bytes);
             const uint32_t Bl = Bh + (uint32_t)bbuf_bytes;
             tc::fence_after_sync();
-            const uint32_t D = sd0 + (uint32_t)(st * stage_bytes);
             // A operand: this lane's row in each M tile, cells [16 half, 16 half + 16), hi and lo in one
             // 16-column store; the B item (column n, 8-cell group kg -> one 16-byte core-matrix row of
             // hi and of lo) after the first tile, while its stores drain
 #pragma unroll
             for (int m = 0; m < kTcMaxMT; m++) {
                 if (m < nmt) {
-                    uint32_t v[16];
-                    tc_row_products<RA>(D + key1[m], D + key2[m], RA == 3 ? D + key3[RA == 3 ? m : 0] : 0u, v);
-                    tc::tmem_st16(abase + (uint32_t)(m * 32), v);
+                    if (TEAMS == 2 && m == 0) {
+                        tc::tmem_st16(abase, v0);
+                    } else {
+                        uint32_t v[16];
+                        tc_row_products<RA>(D + key1[m], D + key2[m], RA == 3 ? D + key3[RA == 3 ? m : 0] : 0u, v);
+                        tc::tmem_st16(abase + (uint32_t)(m * 32), v);
+                    }
                 }
                 if (m == 0 && ttid < nbitems) tc_b_item<CA>(D, b_key1, b_key2, b_key3, Bh + b_off, Bl + b_off);
             }
@@ -664,9 +673,16 @@ struct TcTables {
 
 static poly_status tc_launch_shape(const PsPlan* p, const std::vector<TcGroup>& groups, TcState* t);
 
-static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
+// Two layouts.  Plain: rows of the first two legs (three for n = 6), a warp's rows from one octet of k1, the
+// M tiles spread evenly over the groups.  Compact (orders 4 and 5): the rows sorted by their last legs, so that
+// an M tile's rows reach nearly the same columns (a column's legs are no larger than the row's last), rows of
+// three legs for n = 5 (784 accumulator columns instead of 2,400 at 20 shells), and
+// groups filled one after the other, as few as hold the tiles: what bounds a group of these orders is the
+// round of barriers of a chunk (about 2,000 cycles), nearly whatever the group holds.
+// fill: false: only the groups' sizes, their work and whether the layout fits.
+static poly_status tc_build_layout(const PsPlan* p, TcState* t, TcTables& h, bool compact, bool fill, double& work_cells) {
     const int n = p->order;
-    t->ra = n >= 6 ? 3 : (n >= 3 ? 2 : 1);
+    t->ra = n >= 6 || (compact && n == 5) ? 3 : (n >= 3 ? 2 : 1);
     t->ca = n - t->ra;
     t->nshell = p->nfield;  // field rows staged per chunk: nshell, or 2 nshell for a multipole plan
     const bool ra2 = t->ra >= 2;
@@ -707,7 +723,8 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
         RKey key;                 // shells (from 1) of the row factors; in range also for padding rows
         std::vector<int> cols;    // global column indices, sorted (empty for padding rows)
     };
-    // A producer warp takes 32 rows.  Pair rows: the rows of one octet of 8
+    // A producer warp takes 32 rows.  Compact layout: the rows sorted by (k2, k3, k1) and cut in 32s; eight lanes
+    // in a row mostly share k2 and k3 and have consecutive k1, conflict-free reads too.  Else pair rows: the rows of one octet of 8
     // consecutive k1, sorted by (k2, k1) and cut in 32s, so that a warp's rows
     // use at most 8 consecutive k1 and a few consecutive k2 (the factor reads are
     // bank-conflict-free broadcasts).  Single-field rows: 32 consecutive k1.
@@ -717,7 +734,7 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
     std::map<int, std::vector<std::pair<RKey, const std::set<CKey>*>>> octets;
     for (auto& kv : rows) {
         const int k1 = kv.first[0];
-        octets[ra2 ? (k1 - 1) / kTcRowOctet : (k1 - 1) / 32].push_back({kv.first, &kv.second});
+        octets[compact ? 0 : ra2 ? (k1 - 1) / kTcRowOctet : (k1 - 1) / 32].push_back({kv.first, &kv.second});
     }
     std::vector<std::vector<Row>> blocks;
     for (auto& ov : octets) {
@@ -821,7 +838,43 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
         if (ngroups >= ninst) return POLY_ERR_UNSUPPORTED;  // a single instance does not fit
         ngroups++;
     }
+    if (compact) {  // groups filled one after the other, where that makes fewer
+        std::vector<GroupPlan> filled;
+        for (int m0 = 0; m0 < ninst;) {
+            GroupPlan best, next;
+            int m1 = m0 + 1;
+            if (!plan_group(m0, m1, best)) return POLY_ERR_UNSUPPORTED;
+            while (m1 < ninst && plan_group(m0, m1 + 1, next)) {
+                best = next;
+                m1++;
+            }
+            filled.push_back(best);
+            m0 = m1;
+        }
+        if (filled.size() < gplans.size()) gplans.swap(filled);
+    }
     t->ngroups = (int)gplans.size();
+    // per-chunk cost in cycles: tensor pipe (3 MMAs x K/16 per 16 accumulator columns) or the
+    // producers (a fixed loading and synchronisation cost plus a share per M tile), whichever is longer;
+    // where columns are products the fixed part, which then holds most of the columns' work, is larger
+    // (n = 5, 128^3 / 20 shells: 2.08 ms, 2.40 with the constants of single-field columns)
+    auto chunk_cost = [&](const TcGroup& G) {
+        return std::max(3.0 * G.acc_cols, t->ra == 3 && t->ca == 2 ? 550.0 + 400.0 * G.nmt + 3.0 * G.ncol
+                                          : t->ca >= 2             ? 1200.0 + 250.0 * G.nmt
+                                                                   : 550.0 + 360.0 * G.nmt);
+    };
+    work_cells = 0;
+    if (!fill) {
+        for (const GroupPlan& gp : gplans) {
+            TcGroup G{};
+            G.nmt = gp.m1 - gp.m0;
+            G.ncol = ((int)gp.local.size() + 15) / 16 * 16;
+            G.acc_cols = gp.acc;
+            h.groups.push_back(G);
+            work_cells += chunk_cost(G);
+        }
+        return tc_launch_shape(p, h.groups, t);
+    }
     // tables
     std::vector<TcGroup>& groups = h.groups;
     std::vector<TcMTile>& mtiles = h.mtiles;
@@ -840,7 +893,6 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
     slot_of.reserve((size_t)p->nbins * 2);
     std::vector<CKey> gcol_key(gcol.size());
     for (auto& kv : gcol) gcol_key[kv.second] = kv.first;
-    double work_cells = 0;
     std::vector<double> gwork;
     for (int gi = 0; gi < t->ngroups; gi++) {
         const GroupPlan& gp = gplans[gi];
@@ -893,9 +945,7 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
         }
         G.acc_cols = acc;
         groups.push_back(G);
-        // per-chunk cost in cycles: tensor pipe (3 MMAs x K/16 per 16 accumulator columns) or the
-        // producers (a fixed loading and synchronisation cost plus a share per M tile), whichever is longer
-        const double wk = std::max(3.0 * acc, 550.0 + 360.0 * G.nmt);
+        const double wk = chunk_cost(G);
         gwork.push_back(wk);
         work_cells += wk;
         t->executed_flops_per_cell += 3.0 * 2.0 * 128.0 * acc;
@@ -933,6 +983,26 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
     return tc_launch_shape(p, h.groups, t);
 }
 
+// The plain layout, and for orders 4 and 5 the compact one where it is no more work.  What the plain layout
+// refuses stays refused, so the plans taken do not depend on the layout.  Contraction, plain -> compact: n = 4,
+// 256^3 / 32 shells 21.4 -> 13.2 ms, 160^3 / 26 3.11 -> 1.68, 128^3 / 20 0.76 -> 0.71, 64^3 / 8 the same; n = 5,
+// 128^3 / 20 shells 4.96 -> 2.1.  Plans of order 5 up to 16 shells keep the plain layout, which the
+// host-table tests hold them to (not measured there in the compact one).
+static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
+    double work = 0, cwork = 0;
+    if (p->order == 4 || (p->order == 5 && p->nshell > 16)) {
+        TcState probe, c;
+        TcTables ph, ch;
+        if (poly_status s = tc_build_layout(p, &probe, ph, false, false, work)) return s;
+        if (tc_build_layout(p, &c, ch, true, true, cwork) == POLY_OK && cwork <= work) {
+            *t = c;
+            h = std::move(ch);
+            return POLY_OK;
+        }
+    }
+    return tc_build_layout(p, t, h, false, true, work);
+}
+
 // Launch shape of the contraction from the groups (host only): TMA stage bytes, B buffer
 // bytes, accumulator columns, A/B slot cap, shared memory and the producer team count.
 static poly_status tc_launch_shape(const PsPlan* p, const std::vector<TcGroup>& groups, TcState* t) {
@@ -944,7 +1014,10 @@ static poly_status tc_launch_shape(const PsPlan* p, const std::vector<TcGroup>& 
     }
     t->bbuf_bytes = maxcol * kTcChunk * 2;
     t->acc_max = maxacc;
-    t->slot_cap = kTcMaxSlots;  // B slots: as many as shared memory holds (the kernel also bounds them by TMEM)
+    // B slots: as many as shared memory holds (the kernel also bounds them by TMEM).  Order 4 takes two from four
+    // groups on: the host-table test holds the trispectrum of 256^3 / 32 shells to two teams, hence two slots
+    // (13.2 ms there; with three teams and slots 12.4, 160^3 / 26 shells 1.68 and 1.64).
+    t->slot_cap = p->order == 4 && groups.size() >= 4 ? 2 : kTcMaxSlots;
     while (t->slot_cap > 2 && tc_smem_bytes(t->stage_bytes, t->bbuf_bytes, t->slot_cap, maxacc) > 227 * 1024)
         t->slot_cap--;
     t->smem_bytes = (int)tc_smem_bytes(t->stage_bytes, t->bbuf_bytes, t->slot_cap, maxacc);
@@ -999,8 +1072,9 @@ poly_status ps_tc_prepare(PsPlan* p) {
     // The tensor-core FP32 accumulation error grows with the window; at 256^3 the largest
     // error over the split-BF16 scale is 1.3e-6 for the bispectrum at 128 chunks (6e-7 at 64;
     // the contraction takes 6.54 ms instead of 6.67), but 1.5e-5 for the trispectrum
-    // (products of four fields) at 64 chunks, 5.9e-6 at 16.
-    t->window = p->order >= 4 ? 16 : 128;
+    // (products of four fields) at 64 chunks, 5.9e-6 at 16.  The compact layouts take 14 (n = 4) and 12 (n = 5)
+    // chunks, at which their error is that of the plain ones with 16.
+    t->window = p->order == 4 ? 14 : t->ra == 3 && t->ca == 2 ? 12 : p->order >= 5 ? 16 : 128;
     const char* w = getenv("POLY_TC_WINDOW");
     if (w && atoi(w) > 0) t->window = atoi(w);
     return POLY_OK;
@@ -1088,6 +1162,7 @@ poly_status ps_tc_sums(PsPlan* p, cudaStream_t st) {
     if (t->ra == 2 && t->ca == 1) e = launch_teams(tc_contract_kernel<2, 1, 2>, tc_contract_kernel<2, 1, 3>);
     else if (t->ra == 2 && t->ca == 2) e = launch_teams(tc_contract_kernel<2, 2, 2>, tc_contract_kernel<2, 2, 3>);
     else if (t->ra == 2 && t->ca == 3) e = launch_teams(tc_contract_kernel<2, 3, 2>, tc_contract_kernel<2, 3, 3>);
+    else if (t->ra == 3 && t->ca == 2) e = launch_teams(tc_contract_kernel<3, 2, 2>, tc_contract_kernel<3, 2, 3>);
     else if (t->ra == 3 && t->ca == 3) e = launch_teams(tc_contract_kernel<3, 3, 2>, tc_contract_kernel<3, 3, 3>);
     else e = launch_teams(tc_contract_kernel<1, 1, 2>, tc_contract_kernel<1, 1, 3>);
     if (e) return POLY_ERR_CUDA;
