@@ -1,7 +1,11 @@
 // Warp-level mixed-radix Stockham FFT over lines held in (padded) shared memory.
 //
 // A line of length N is transformed in place, X[k] = sum_j x[j] e^{SIGN 2 pi i jk/N}
-// (unnormalised).  Radices are 16 first, then 8, 4, 2, 3, 5; stage s with radix R
+// (unnormalised).  Radices are 16 first, then 8, 4, 2, 3, 5, except that 96 = 12 x 8 and
+// single-precision 160 = 16 x 10 take two stages instead of three (16 x 2 x 3 and
+// 16 x 2 x 5).  In double precision 160 keeps three: its second stage would leave a
+// quarter of the lanes idle, and FP64 issue is what bounds it (32 fields of 160^3: 4.56 ms
+// with three stages, 4.93 with two; 31 of 96^3: 1.25 and 1.06); stage s with radix R
 // and Ns = product of earlier radices maps butterfly j (0 <= j < N/R):
 //   v[r] = x[j + r N/R] * W_{Ns R}^{SIGN (j mod Ns) r},  V = DFT_R(v),
 //   y[(j / Ns) Ns R + (j mod Ns) + r Ns] = V[r].
@@ -15,14 +19,17 @@
 namespace ps {
 
 // ---- radix plan (compile time) --------------------------------------------
-__host__ __device__ constexpr int fft_nstages(int n) {
+__host__ __device__ constexpr bool fft_two_stages(int n, bool fp64) { return n == 96 || (n == 160 && !fp64); }
+__host__ __device__ constexpr int fft_nstages(int n, bool fp64) {
+    if (fft_two_stages(n, fp64)) return 2;
     int s = 0;
     while (n % 16 == 0) { n /= 16; s++; }
     for (int r : {8, 4, 2, 3, 5})
         while (n % r == 0) { n /= r; s++; }
     return n == 1 ? s : -1;
 }
-__host__ __device__ constexpr int fft_radix(int n, int stage) {
+__host__ __device__ constexpr int fft_radix(int n, int stage, bool fp64) {
+    if (fft_two_stages(n, fp64)) return stage == 0 ? (n == 96 ? 12 : 16) : stage == 1 ? (n == 96 ? 8 : 10) : 1;
     int s = 0;
     while (n % 16 == 0) {
         if (s == stage) return 16;
@@ -37,14 +44,14 @@ __host__ __device__ constexpr int fft_radix(int n, int stage) {
         }
     return 1;
 }
-__host__ __device__ constexpr int fft_ns(int n, int stage) {  // product of radices before `stage`
+__host__ __device__ constexpr int fft_ns(int n, int stage, bool fp64) {  // product of radices before `stage`
     int p = 1;
-    for (int s = 0; s < stage; s++) p *= fft_radix(n, s);
+    for (int s = 0; s < stage; s++) p *= fft_radix(n, s, fp64);
     return p;
 }
-// lines per warp: enough butterflies in the first stage to occupy the lanes
+// lines per warp: enough butterflies in the first stage (the same in both precisions) to occupy the lanes
 __host__ __device__ constexpr int fft_lpw(int n) {
-    int b = n / fft_radix(n, 0);
+    int b = n / fft_radix(n, 0, false);
     int l = 32 / b;
     return l < 1 ? 1 : l;
 }
@@ -150,6 +157,42 @@ PS_DEV void dft16(Cx<T>* v) {
     for (int i = 0; i < 16; i++) v[i] = t[i];
 }
 
+// Lengths 10 = 2 x 5 and 12 = 3 x 4 with coprime factors (Good's prime-factor map): input n = (5 n1 + 2 n2) mod 10
+// or (4 n1 + 3 n2) mod 12 turns the sum into a two-dimensional transform without twiddles, whose value at
+// (k mod 2, k mod 5) or (k mod 3, k mod 4) is X[k].
+template <typename T, int SIGN>
+PS_DEV void dft10(Cx<T>* v) {
+    Cx<T> y[2][5];
+#pragma unroll
+    for (int n2 = 0; n2 < 5; n2++) {
+        const Cx<T> a = v[(2 * n2) % 10], b = v[(5 + 2 * n2) % 10];
+        y[0][n2] = cadd(a, b);
+        y[1][n2] = csub(a, b);
+    }
+    dft5<T, SIGN>(y[0]);
+    dft5<T, SIGN>(y[1]);
+#pragma unroll
+    for (int k = 0; k < 10; k++) v[k] = y[k % 2][k % 5];
+}
+
+template <typename T, int SIGN>
+PS_DEV void dft12(Cx<T>* v) {
+    Cx<T> y[3][4];
+#pragma unroll
+    for (int n2 = 0; n2 < 4; n2++) {
+        Cx<T> t[3];
+#pragma unroll
+        for (int n1 = 0; n1 < 3; n1++) t[n1] = v[(4 * n1 + 3 * n2) % 12];
+        dft3<T, SIGN>(t);
+#pragma unroll
+        for (int k1 = 0; k1 < 3; k1++) y[k1][n2] = t[k1];
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; k1++) dft4<T, SIGN>(y[k1][0], y[k1][1], y[k1][2], y[k1][3]);
+#pragma unroll
+    for (int k = 0; k < 12; k++) v[k] = y[k % 3][k % 4];
+}
+
 template <typename T, int R, int SIGN>
 PS_DEV void dft(Cx<T>* v) {
     if constexpr (R == 2) dft2<T, SIGN>(v);
@@ -157,6 +200,8 @@ PS_DEV void dft(Cx<T>* v) {
     else if constexpr (R == 4) dft4<T, SIGN>(v[0], v[1], v[2], v[3]);
     else if constexpr (R == 5) dft5<T, SIGN>(v);
     else if constexpr (R == 8) dft8<T, SIGN>(v);
+    else if constexpr (R == 10) dft10<T, SIGN>(v);
+    else if constexpr (R == 12) dft12<T, SIGN>(v);
     else if constexpr (R == 16) dft16<T, SIGN>(v);
 }
 
@@ -173,9 +218,10 @@ struct SmemLines {
 template <typename T, int N, int STAGE, int SIGN, int LPW, class Reader, class Writer>
 PS_DEV void fft_stage(const SmemLines<T>& buf, int nl, const Cx<T>* tw, int lane, const Reader& rd,
                       const Writer& wr) {
-    constexpr int NST = fft_nstages(N);
-    constexpr int R = fft_radix(N, STAGE);
-    constexpr int NS = fft_ns(N, STAGE);
+    constexpr bool FP64 = sizeof(T) == 8;
+    constexpr int NST = fft_nstages(N, FP64);
+    constexpr int R = fft_radix(N, STAGE, FP64);
+    constexpr int NS = fft_ns(N, STAGE, FP64);
     constexpr int B = N / R;
     constexpr int TOT = LPW * B;
     constexpr int CNT = (TOT + 31) / 32;
@@ -219,7 +265,7 @@ PS_DEV void fft_stage(const SmemLines<T>& buf, int nl, const Cx<T>* tw, int lane
 template <typename T, int N, int STAGE, int SIGN, int LPW, class Reader, class Writer>
 PS_DEV void fft_stages(const SmemLines<T>& buf, int nl, const Cx<T>* tw, int lane, const Reader& rd,
                        const Writer& wr) {
-    if constexpr (STAGE < fft_nstages(N)) {
+    if constexpr (STAGE < fft_nstages(N, sizeof(T) == 8)) {
         fft_stage<T, N, STAGE, SIGN, LPW>(buf, nl, tw, lane, rd, wr);
         fft_stages<T, N, STAGE + 1, SIGN, LPW>(buf, nl, tw, lane, rd, wr);
     }
@@ -230,7 +276,7 @@ PS_DEV void fft_stages(const SmemLines<T>& buf, int nl, const Cx<T>* tw, int lan
 template <typename T, int N, int SIGN, class Reader, class Writer>
 PS_DEV void warp_fft(const SmemLines<T>& buf, int nl, const Cx<T>* tw, int lane, const Reader& rd,
                      const Writer& wr) {
-    static_assert(fft_nstages(N) > 0, "unsupported FFT length");
+    static_assert(fft_nstages(N, sizeof(T) == 8) > 0, "unsupported FFT length");
     fft_stages<T, N, 0, SIGN, fft_lpw(N)>(buf, nl, tw, lane, rd, wr);
 }
 

@@ -21,6 +21,28 @@ constexpr int kPlaneThreads = 256;
 constexpr int kPlaneWarps = kPlaneThreads / 32;
 constexpr int kXLines = 32;  // lines per block in the x pass
 
+// Stride of the row buffers that a warp transforms: line l's B = N / (first radix) butterflies start at l * stride,
+// so a stride of B (mod the 16 or 8 complex values of 128 bytes) gives the lanes of a first-stage access
+// consecutive positions (two to three accesses to a bank with the column stride of line_stride).  With the
+// stages of 96 and 160 (fft_radix) and the blocks of SmallPlane below: the 31 shells of 96^3 take 82 us of
+// inverse planes instead of 225, the 32 fields of 160^3 0.270 ms instead of 0.383 (FP32).
+template <typename T, int N>
+PS_HD constexpr int row_stride() {
+    constexpr int m = (int)(128 / (2 * sizeof(T))), B = N / fft_radix(N, 0, sizeof(T) == 8);
+    int s = N + N / m;
+    while (s % m != B % m) s++;
+    return s;
+}
+
+// Blocks of the shells whose plane buffer fits several times per SM: warps, and blocks per SM that the registers
+// must allow.  The warps divide the groups of row pairs that a warp transforms at a time: 96: 12 groups over 4
+// warps (8 leave a third of the second round idle), 64: 4 over 4, 160: 27 over 9.
+template <int N>
+struct SmallPlane {
+    static constexpr int warps = N == 96 || N == 64 ? 4 : N == 160 ? 9 : 8;
+    static constexpr int blocks = N == 96 || N == 64 ? 4 : 2;
+};
+
 template <typename T>
 PS_DEV void load_twiddles(Cx<T>* s_tw, const Cx<double>* g_tw, int n) {
     for (int m = threadIdx.x; m < n; m += blockDim.x) s_tw[m] = cx<T>((T)g_tw[m].re, (T)g_tw[m].im);
@@ -51,8 +73,9 @@ __global__ void __launch_bounds__(kPlaneThreads) fwd_plane_kernel(const T* __res
     const int ls = line_stride<T>(N);
     constexpr int LPW = fft_lpw(N);
     Cx<T>* s_tw = reinterpret_cast<Cx<T>*>(smem_raw);
+    constexpr int zs = row_stride<T, N>();
     Cx<T>* s_z = s_tw + N;                              // per-warp row buffers
-    Cx<T>* s_t = s_z + (size_t)kPlaneWarps * LPW * ls;  // (K+1) lines of ls
+    Cx<T>* s_t = s_z + (size_t)kPlaneWarps * LPW * zs;  // (K+1) lines of ls
     const int x = blockIdx.x;
     // blockIdx.y: the field of a batch (fields N^3 apart, their W outputs N (2K+1)(K+1) apart)
     delta += (size_t)blockIdx.y * N * N * N;
@@ -63,7 +86,7 @@ __global__ void __launch_bounds__(kPlaneThreads) fwd_plane_kernel(const T* __res
     __syncthreads();
 
     const T* plane = delta + (size_t)x * N * N;
-    SmemLines<T> zb{s_z + (size_t)warp * LPW * ls, ls};
+    SmemLines<T> zb{s_z + (size_t)warp * LPW * zs, zs};
     const int npairs = (N + 1) / 2;
     for (int p0 = warp * LPW; p0 < npairs; p0 += kPlaneWarps * LPW) {
         const int nl = min(LPW, npairs - p0);
@@ -285,8 +308,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) inv_plane_kernel(
     const int ls = line_stride<T>(N);
     constexpr int LPW = fft_lpw(N);
     Cx<T>* s_tw = reinterpret_cast<Cx<T>*>(smem_raw);
+    constexpr int zs = row_stride<T, N>();
     Cx<T>* s_z = s_tw + N;
-    Cx<T>* s_h = s_z + (size_t)WARPS * LPW * ls;
+    Cx<T>* s_h = s_z + (size_t)WARPS * LPW * zs;
     const int x = x0 + blockIdx.x;
     const int s = s0 + blockIdx.y;
     Cx<T>* Hb = SPILL ? spill + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (size_t)(K + 1) * ls : s_h;
@@ -379,7 +403,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) inv_plane_kernel(
     __syncthreads();
     // real transform along z, two rows per complex line, written straight to global
     T* plane = out + (size_t)(s - plane_s0) * out_shell_stride + (size_t)blockIdx.x * N * N;
-    SmemLines<T> zb{s_z + (size_t)warp * LPW * ls, ls};
+    SmemLines<T> zb{s_z + (size_t)warp * LPW * zs, zs};
     const int npairs = (N + 1) / 2;
     for (int p0 = warp * LPW; p0 < npairs; p0 += WARPS * LPW) {
         const int nl = min(LPW, npairs - p0);
@@ -395,7 +419,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) inv_plane_kernel(
 template <typename T, int N>
 static size_t plane_smem_n(int K, bool spill, int warps = kPlaneWarps) {
     const int ls = line_stride<T>(N);
-    size_t e = N + (size_t)warps * fft_lpw(N) * ls + (spill ? 0 : (size_t)(K + 1) * ls);
+    size_t e = N + (size_t)warps * fft_lpw(N) * row_stride<T, N>() + (spill ? 0 : (size_t)(K + 1) * ls);
     return e * sizeof(Cx<T>);
 }
 
@@ -475,8 +499,8 @@ static cudaError_t inverse_n(const Cx<T>* fhat, const short4* lines, const int* 
 
 // The inverse for the estimate path (FP32, natural or tiled output, x pass in
 // front) in runs of consecutive shells, each launched with the shared memory
-// its own largest kz needs: shells whose plane buffer fits twice per SM run as
-// 8-warp blocks, two per SM, so that one block's transform phases overlap the
+// its own largest kz needs: shells whose plane buffer fits several times per SM
+// run as small blocks (SmallPlane), so that one block's transform phases overlap the
 // other's; the rest run as one 16-warp block per SM.  kz_host[s] is shell s's
 // largest kz (host array), kz_dev the same table on the device (or NULL).
 template <typename T, int N>
@@ -492,20 +516,21 @@ static cudaError_t inverse_ranged_n(const Cx<T>* fhat, const short4* lines, cons
     if ((e = cudaFuncSetAttribute(kx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smx))) return e;
     kx<<<dim3((max_lines + 31) / 32, ns), 256, smx, st>>>(fhat, lines, line_off, s0, K, tw_inv, xpre);
     if ((e = cudaGetLastError())) return e;
-    // largest kz whose 8-warp block fits twice per SM (228 KB per SM, 1 KB reserved per block)
-    constexpr size_t kHalfSm = 228 * 1024 / 2 - 1024;
+    // largest kz whose small block fits often enough per SM (228 KB per SM, 1 KB reserved per block)
+    using SP = SmallPlane<N>;
+    constexpr size_t kShare = 228 * 1024 / SP::blocks - 1024;
     int ksmall = -1;
-    while (ksmall < K && plane_smem_n<T, N>(ksmall + 1, false, 8) <= kHalfSm) ksmall++;
+    while (ksmall < K && plane_smem_n<T, N>(ksmall + 1, false, SP::warps) <= kShare) ksmall++;
     for (int r0 = s0; r0 < s0 + ns;) {
         const bool small = kz_host[r0] <= ksmall;
         int r1 = r0 + 1, kzm = kz_host[r0];
         while (r1 < s0 + ns && (kz_host[r1] <= ksmall) == small) kzm = std::max(kzm, kz_host[r1++]);
         const dim3 grid(N, r1 - r0);
         if (small) {
-            auto k = inv_plane_kernel<T, N, false, false, true, 8, 2>;
-            const size_t sm = plane_smem_n<T, N>(kzm, false, 8);
+            auto k = inv_plane_kernel<T, N, false, false, true, SP::warps, SP::blocks>;
+            const size_t sm = plane_smem_n<T, N>(kzm, false, SP::warps);
             if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-            k<<<grid, 8 * 32, sm, st>>>(fhat, lines, line_off, r0, K, 0, tw_inv, out, out_stride, nullptr, xpre, tile_ns,
+            k<<<grid, SP::warps * 32, sm, st>>>(fhat, lines, line_off, r0, K, 0, tw_inv, out, out_stride, nullptr, xpre, tile_ns,
                                         s0, kz_dev);
         } else {
             auto k = inv_plane_kernel<T, N, false, false, true, 16, 1>;
