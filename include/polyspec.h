@@ -78,7 +78,7 @@ typedef enum {
  * drawn from, C(nshell + n - 1, n) of them, may number at most 2^26
  * (POLY_ERR_UNSUPPORTED above; e.g. n = 5 with 120 shells).  Argument checks
  * and the host tables come before any device call.  Plan creation enumerates the bins,
- * builds the shell tables and tiles, allocates the workspace (nshell * N^3
+ * builds the shell tables and the contraction's tasks, allocates the workspace (nshell * N^3
  * fields of the plan's precision plus small buffers) on the current CUDA
  * device and computes the exact counts (FP64 counting fields on the
  * 1/48 symmetry wedge, cached per (N, edges, n, flags) in the process).  Where
@@ -309,8 +309,8 @@ typedef struct {
     float ms_forward;   /* last timed estimate: forward R2C transform */
     float ms_fields;    /* last timed estimate: shell gather + inverse transforms (all shells) */
     float ms_contract;  /* last timed estimate: the product-sum contraction kernel */
-    float ms_reduce;    /* last timed estimate: cross-tile reduction + normalisation */
-    double contract_flops; /* flops the contraction kernel executes per estimate (dense tiles; the tensor
+    float ms_reduce;    /* last timed estimate: reduction over the blocks + normalisation (one kernel) */
+    double contract_flops; /* flops the contraction kernel executes per estimate (whole register blocks; the tensor
                               path counts its three split products) */
 } poly_stats;
 

@@ -65,6 +65,13 @@ PS_HD Cx<T> cscale(Cx<T> a, T s) { return cx<T>(a.re * s, a.im * s); }
 template <int SIGN, typename T>
 PS_HD Cx<T> cmul_si(Cx<T> a) { return SIGN > 0 ? cx<T>(-a.im, a.re) : cx<T>(a.im, -a.re); }
 
+// Sum over the warp's lanes, in a fixed order (the result in every lane).
+PS_DEV double warp_sum(double s) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    return s;
+}
+
 // Shared-memory index padded with one element per 128 bytes, so that the
 // Stockham write pattern (stride = radix) and strided column reads spread
 // over the 32 banks.

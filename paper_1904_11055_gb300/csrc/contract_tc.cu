@@ -509,14 +509,22 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
     if (tid == 0 && *s_abort) atomicExch(err, tc::kErrTimeout);
 }
 
-// S[b] = sum over the blocks of the bin's group of partial[block][slot]
-__global__ void tc_reduce_kernel(const double* __restrict__ partial, const int4* __restrict__ bin_map, int64_t nbins,
-                                 double* __restrict__ S) {
-    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nbins; b += (int64_t)gridDim.x * blockDim.x) {
+// out[b] = norm * S_b / (n3 count_b) (0 where the count is 0), S_b = the sum over the blocks of the bin's group of
+// partial[block][slot]; one warp per bin (see reduce_slots_kernel)
+__global__ void tc_reduce_kernel(const double* __restrict__ partial, const int4* __restrict__ bin_map,
+                                 const int64_t* __restrict__ counts, int64_t nbins, double norm, double n3,
+                                 double* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t b = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); b < nbins; b += nw) {
         const int4 m = bin_map[b];  // first block, block count, slot
         double s = 0.0;
-        for (int k = 0; k < m.y; k++) s += partial[(size_t)(m.x + k) * (kTcAccMax * 128) + m.z];
-        S[b] = s;
+        for (int k = lane; k < m.y; k += 32) s += partial[(size_t)(m.x + k) * (kTcAccMax * 128) + m.z];
+        s = warp_sum(s);
+        if (lane == 0) {
+            const int64_t c = counts[b];
+            out[b] = c > 0 ? norm * s / (n3 * (double)c) : 0.0;
+        }
     }
 }
 
@@ -1145,7 +1153,7 @@ extern "C" int poly_diag_tc_tables(int N, int order, const double* edges, int ns
     }
 }
 
-poly_status ps_tc_sums(PsPlan* p, cudaStream_t st) {
+poly_status ps_tc_sums(PsPlan* p, double norm, double* out, cudaStream_t st) {
     TcState* t = p->tc;
     if (!t) return POLY_ERR_UNSUPPORTED;
     cudaError_t e;
@@ -1167,8 +1175,9 @@ poly_status ps_tc_sums(PsPlan* p, cudaStream_t st) {
     else e = launch_teams(tc_contract_kernel<1, 1, 2>, tc_contract_kernel<1, 1, 3>);
     if (e) return POLY_ERR_CUDA;
     if (p->timing) cudaEventRecord(p->ev[3], st);
-    const int blocks = (int)std::min<int64_t>((p->nbins + 255) / 256, 4096);
-    tc_reduce_kernel<<<std::max(1, blocks), 256, 0, st>>>(t->d_partial, (const int4*)t->d_binmap, p->nbins, p->d_S);
+    const int blocks = (int)std::min<int64_t>((p->nbins + 7) / 8, 8192);
+    tc_reduce_kernel<<<std::max(1, blocks), 256, 0, st>>>(t->d_partial, (const int4*)t->d_binmap, p->d_counts, p->nbins, norm,
+                                                          (double)p->N * p->N * p->N, out);
     p->launches += 2;
     return cudaGetLastError() ? POLY_ERR_CUDA : POLY_OK;
 }

@@ -90,18 +90,15 @@ struct CcLaunch {
 cudaError_t ps_contract_cc(int is_double, int order, int weighted, int absval, const CcLaunch& L, const void* fields,
                            const void* weight, const CcGroup* groups, const CcTask* tasks, double* partial,
                            cudaStream_t st);
-// S[b] = sum_split partial[split * slot_stride + slot[b]]
+// out[b] = norm * S_b / (n3 count[b]) (0 where count == 0; counts NULL: S_b), S_b = sum_split partial[split * slot_stride + slot[b]]
 cudaError_t ps_reduce_slots(const double* partial, int nsplit, int64_t slot_stride, const int64_t* slot,
-                            int64_t nbins, double* S, cudaStream_t st);
-// out[b] = norm * S[b] / (N^3 count[b])  (0 where count == 0)
+                            const int64_t* counts, int64_t nbins, double norm, double n3, double* out, cudaStream_t st);
 // disconnected part of the trispectrum: shell powers P (device, nshell) from the pruned spectrum, then B_disc per bin
 cudaError_t ps_disconnected(int is_double, const void* fhat, const void* lines, const int* line_off, int nshell, int K,
                             const int32_t* bins, const int64_t* counts, int64_t nbins, double norm, double n3,
                             double* P, double* out, cudaStream_t st);
 // out = L_ell(kz/|q|) * fhat over the pruned half spectrum (even ell; the mode q = 0 gets weight 0)
 cudaError_t ps_legendre_weight(int is_double, const void* fhat, int K, int ell, void* out, cudaStream_t st);
-cudaError_t ps_normalise(const double* S, const int64_t* counts, int64_t nbins, double norm, double n3, double* out,
-                         cudaStream_t st);
 
 // ---- misc.cu -------------------------------------------------------------------
 // ---- counts_exact.cu ---------------------------------------------------------

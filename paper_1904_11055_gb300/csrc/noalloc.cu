@@ -189,7 +189,7 @@ static poly_status estimate_noalloc(int N, double L, int nshell, const double* e
     const size_t o_groups = c.take(hp.cc.groups.size() * sizeof(CcGroup));
     const size_t o_slot = c.take(hp.cc.slot.size() * sizeof(int64_t));
     const size_t o_part = c.take((size_t)(cl.rows() * cl.stride()) * 8);
-    const size_t o_S = c.take((size_t)hp.nbins * 8), o_cnt = c.take((size_t)hp.nbins * 8);
+    const size_t o_cnt = c.take((size_t)hp.nbins * 8);
     if (c.used > kNoAllocBytes)
         return fail(POLY_ERR_UNSUPPORTED, "this problem needs " + std::to_string(c.used >> 20) +
                                               " MiB of scratch; the static array holds 32 MiB");
@@ -225,19 +225,17 @@ static poly_status estimate_noalloc(int N, double L, int nshell, const double* e
             cudaError_t e = cudaMemcpyAsync(B + cp.off, cp.src, cp.bytes, cudaMemcpyHostToDevice, st);
             if (e) return fail(POLY_ERR_CUDA, std::string("copy into scratch: ") + cudaGetErrorString(e));
         }
+    const double n3d = (double)n3;
+    const double norm = std::pow(L * L * L, order - 1) / std::pow(n3d, order);
     cudaError_t e;
     if ((e = ps_forward(N, 0, delta_x, K, B + o_twf, B + o_W, B + o_fhat, nullptr, st)) ||
         (e = ps_inverse(N, 0, 0, B + o_fhat, B + o_lines, (const int*)(B + o_loff), 0, nshell, K, 0, N, B + o_twi,
                         B + o_fields, (size_t)n3, nullptr, nullptr, 0, nshell, st)) ||
         (e = ps_contract_cc(0, order, 0, 0, cl, B + o_fields, nullptr, (const CcGroup*)(B + o_groups),
                             (const CcTask*)(B + o_tasks), (double*)(B + o_part), st)) ||
-        (e = ps_reduce_slots((const double*)(B + o_part), (int)cl.rows(), cl.stride(), (const int64_t*)(B + o_slot), hp.nbins,
-                             (double*)(B + o_S), st)))
+        (e = ps_reduce_slots((const double*)(B + o_part), (int)cl.rows(), cl.stride(), (const int64_t*)(B + o_slot),
+                             (const int64_t*)(B + o_cnt), hp.nbins, norm, n3d, out, st)))
         return fail(POLY_ERR_CUDA, std::string("estimate kernels: ") + cudaGetErrorString(e));
-    const double n3d = (double)n3;
-    const double norm = std::pow(L * L * L, order - 1) / std::pow(n3d, order);
-    if ((e = ps_normalise((const double*)(B + o_S), (const int64_t*)(B + o_cnt), hp.nbins, norm, n3d, out, st)))
-        return fail(POLY_ERR_CUDA, std::string("normalise: ") + cudaGetErrorString(e));
     return POLY_OK;
 }
 

@@ -1,5 +1,5 @@
 // Host side of the polyspectrum library: plan construction (shell tables, bin
-// enumeration, contraction tiles, exact counts) and the C ABI of polyspec.h.
+// enumeration, contraction tasks, exact counts) and the C ABI of polyspec.h.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -520,8 +520,8 @@ static poly_status compute_counts(PsPlan* p, cudaStream_t st) {
         if (p->nbins > 0 &&
             ((e = ps_contract_cc(1, p->order, 1, 0, L, d_iota, d_wgt, (const CcGroup*)d_groups, (const CcTask*)d_tasks,
                                  (double*)d_part, st)) ||
-             (e = ps_reduce_slots((double*)d_part, (int)L.rows(), L.stride(), (const int64_t*)d_slot, p->nbins,
-                                  (double*)d_S, st)))) {
+             (e = ps_reduce_slots((double*)d_part, (int)L.rows(), L.stride(), (const int64_t*)d_slot, nullptr, p->nbins,
+                                  1.0, 1.0, (double*)d_S, st)))) {
             rc = cuda_error(e, "count contraction");
             break;
         }
@@ -700,7 +700,6 @@ static poly_status create_plan(PsPlan* p, int N, double L, int order, int nshell
         PS_TRY(ps_alloc(p, &p->d_spill, ps_spill_elems(N, K, N * nshell, p->is_double) * 2 * es));
     p->ccl = cc_launch_shape(p->cc, order, p->nfield, (int64_t)n3 / 32, p->sms);  // N^3 is a multiple of 32 for every N
     PS_TRY(ps_alloc(p, (void**)&p->d_partial, (size_t)(p->ccl.rows() * p->ccl.stride()) * 8));
-    PS_TRY(ps_alloc(p, (void**)&p->d_S, (size_t)std::max<int64_t>(1, p->nbins) * 8));
     PS_TRY(ps_alloc(p, (void**)&p->d_counts, (size_t)std::max<int64_t>(1, p->nbins) * 8));
     PS_TRY(ps_alloc(p, &p->d_in_stage, n3 * es));
     PS_TRY(ps_alloc(p, (void**)&p->d_out_stage, (size_t)std::max<int64_t>(1, p->nbins) * 8));
@@ -763,15 +762,16 @@ poly_status ps_fields(PsPlan* p, const void* delta, cudaStream_t st) {
     return POLY_OK;
 }
 
-poly_status ps_sums(PsPlan* p, bool absval, cudaStream_t st) {
+poly_status ps_sums(PsPlan* p, bool absval, double norm, double* out, cudaStream_t st) {
     cudaError_t e;
-    if (p->prec == POLY_SPLIT_BF16 && !absval) return ps_tc_sums(p, st);
+    if (p->prec == POLY_SPLIT_BF16 && !absval) return ps_tc_sums(p, norm, out, st);
+    const double n3 = (double)p->N * p->N * p->N;
     if ((e = ps_contract_cc(p->is_double, p->order, 0, absval ? 1 : 0, p->ccl, p->d_fields, nullptr,
                             (const CcGroup*)p->d_cc_groups, (const CcTask*)p->d_cc_tasks, p->d_partial, st)))
         return cuda_error(e, "contraction");
     if (!absval) mark(p, 3, st);
-    if ((e = ps_reduce_slots(p->d_partial, (int)p->ccl.rows(), p->ccl.stride(), (const int64_t*)p->d_cc_slot, p->nbins,
-                             p->d_S, st)))
+    if ((e = ps_reduce_slots(p->d_partial, (int)p->ccl.rows(), p->ccl.stride(), (const int64_t*)p->d_cc_slot, p->d_counts,
+                             p->nbins, norm, n3, out, st)))
         return cuda_error(e, "contraction");
     p->launches += 2;
     return POLY_OK;
@@ -784,18 +784,11 @@ double ps_norm(const PsPlan* p) {  // c_n, times 2 ell + 1 for a multipole plan
 
 poly_status ps_estimate_impl(PsPlan* p, const void* delta, double* out, double* scale, cudaStream_t st) {
     PS_TRY(ps_fields(p, delta, st));
-    PS_TRY(ps_sums(p, false, st));
-    const double n3 = (double)p->N * p->N * p->N;
-    cudaError_t e;
-    if ((e = ps_normalise(p->d_S, p->d_counts, p->nbins, ps_norm(p), n3, out, st)))
-        return cuda_error(e, "normalise");
-    p->launches += 1;
+    PS_TRY(ps_sums(p, false, ps_norm(p), out, st));
     mark(p, 4, st);
     if (p->timing) p->ev_recorded = true;
     if (scale) {
-        PS_TRY(ps_sums(p, true, st));
-        if ((e = ps_normalise(p->d_S, p->d_counts, p->nbins, 1.0, n3, scale, st))) return cuda_error(e, "scale");
-        p->launches += 1;
+        PS_TRY(ps_sums(p, true, 1.0, scale, st));
     }
     return POLY_OK;
 }
@@ -1211,9 +1204,9 @@ poly_status poly_plan_tune(poly_plan p, const void* delta_x, int* config_out, do
                 break;
             }
             cudaError_t e = cudaSuccess;
-            if ((s = ps_tc_sums(p, st))) break;  // warm-up
+            if ((s = ps_tc_sums(p, ps_norm(p), p->d_out_stage, st))) break;  // warm-up
             if ((e = cudaEventRecord(e0, st))) s = cuda_error(e, "cudaEventRecord");
-            for (int r = 0; r < 3 && !s; r++) s = ps_tc_sums(p, st);
+            for (int r = 0; r < 3 && !s; r++) s = ps_tc_sums(p, ps_norm(p), p->d_out_stage, st);
             if (!s && (e = cudaEventRecord(e1, st))) s = cuda_error(e, "cudaEventRecord");
             if (!s && (e = cudaEventSynchronize(e1))) s = cuda_error(e, "cudaEventSynchronize");
             if (!s) s = ps_check_device_error(p);

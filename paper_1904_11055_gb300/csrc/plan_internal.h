@@ -70,7 +70,6 @@ struct poly_plan_s {
     void* d_fields = nullptr;  // nshell x N^3 real
     void* d_spill = nullptr;   // plane-kernel overflow (FP64 at large K)
     double* d_partial = nullptr;
-    double* d_S = nullptr;
     int64_t* d_counts = nullptr;
     void* d_in_stage = nullptr;    // host-buffer entry point staging
     double* d_out_stage = nullptr;
@@ -118,13 +117,14 @@ poly_status ps_plan_host_tables(PsPlan* p, int N, double L, int order, int nshel
 poly_status ps_fields(PsPlan* p, const void* delta, cudaStream_t st);
 // true when the x-pass buffer holds shells [s0, s0 + ns) (global line offsets)
 bool ps_xpre_fits(const PsPlan* p, int s0, int ns);
-poly_status ps_sums(PsPlan* p, bool absval, cudaStream_t st);
+// out = norm * S_b / (N^3 count_b) (absval: of the absolute products)
+poly_status ps_sums(PsPlan* p, bool absval, double norm, double* out, cudaStream_t st);
 poly_status ps_estimate_impl(PsPlan* p, const void* delta, double* out, double* scale, cudaStream_t st);
 double ps_norm(const PsPlan* p);
 
 // contract_tc.cu
 poly_status ps_tc_prepare(PsPlan* p);
-poly_status ps_tc_sums(PsPlan* p, cudaStream_t st);
+poly_status ps_tc_sums(PsPlan* p, double norm, double* out, cudaStream_t st);
 void ps_tc_free(PsPlan* p);
 double ps_tc_executed_flops(const PsPlan* p);
 poly_status ps_check_device_error(PsPlan* p);
