@@ -65,17 +65,17 @@ struct RowPairReader {  // Z(z) = delta(x, y1, z) + i delta(x, y2, z)
     }
 };
 
-template <typename T, int N, bool SPILL>
-__global__ void __launch_bounds__(kPlaneThreads) fwd_plane_kernel(const T* __restrict__ delta, int K,
-                                                                  const Cx<double>* __restrict__ g_tw,
-                                                                  Cx<T>* __restrict__ W, Cx<T>* __restrict__ spill) {
+template <typename T, int N, bool SPILL, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32) fwd_plane_kernel(const T* __restrict__ delta, int K,
+                                                               const Cx<double>* __restrict__ g_tw,
+                                                               Cx<T>* __restrict__ W, Cx<T>* __restrict__ spill) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int ls = line_stride<T>(N);
     constexpr int LPW = fft_lpw(N);
     Cx<T>* s_tw = reinterpret_cast<Cx<T>*>(smem_raw);
     constexpr int zs = row_stride<T, N>();
     Cx<T>* s_z = s_tw + N;                              // per-warp row buffers
-    Cx<T>* s_t = s_z + (size_t)kPlaneWarps * LPW * zs;  // (K+1) lines of ls
+    Cx<T>* s_t = s_z + (size_t)WARPS * LPW * zs;  // (K+1) lines of ls
     const int x = blockIdx.x;
     // blockIdx.y: the field of a batch (fields N^3 apart, their W outputs N (2K+1)(K+1) apart)
     delta += (size_t)blockIdx.y * N * N * N;
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kPlaneThreads) fwd_plane_kernel(const T* __res
     const T* plane = delta + (size_t)x * N * N;
     SmemLines<T> zb{s_z + (size_t)warp * LPW * zs, zs};
     const int npairs = (N + 1) / 2;
-    for (int p0 = warp * LPW; p0 < npairs; p0 += kPlaneWarps * LPW) {
+    for (int p0 = warp * LPW; p0 < npairs; p0 += WARPS * LPW) {
         const int nl = min(LPW, npairs - p0);
         RowPairReader<T> rd{plane, 2 * p0, N, N};
         warp_fft<T, N, -1>(zb, nl, s_tw, lane, rd, zb);
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kPlaneThreads) fwd_plane_kernel(const T* __res
     }
     __syncthreads();
     // DFT along y of the K+1 kz columns
-    for (int g = warp * LPW; g <= K; g += kPlaneWarps * LPW) {
+    for (int g = warp * LPW; g <= K; g += WARPS * LPW) {
         SmemLines<T> tb{Tb + (size_t)g * ls, ls};
         warp_fft_inplace<T, N, -1>(tb, min(LPW, K + 1 - g), s_tw, lane);
     }
@@ -435,20 +435,26 @@ constexpr size_t kMaxSmem = 227 * 1024;
 template <typename T, int N>
 static cudaError_t forward_n(const T* delta, int K, const Cx<double>* tw_fwd, Cx<T>* W, Cx<T>* fhat, Cx<T>* spill,
                              cudaStream_t st, int nfields = 1) {
-    bool spill_on = plane_smem_n<T, N>(K, false) > kMaxSmem;
+    const size_t sm8 = plane_smem_n<T, N>(K, false);
+    const bool spill_on = sm8 > kMaxSmem;
     if (spill_on && !spill) return cudaErrorInvalidValue;
-    size_t sm = plane_smem_n<T, N>(K, spill_on);
-    cudaError_t e;
-    if (spill_on) {
-        auto k = fwd_plane_kernel<T, N, true>;
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        k<<<dim3(N, nfields), kPlaneThreads, sm, st>>>(delta, K, tw_fwd, W, spill);
-    } else {
-        auto k = fwd_plane_kernel<T, N, false>;
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        k<<<dim3(N, nfields), kPlaneThreads, sm, st>>>(delta, K, tw_fwd, W, nullptr);
-    }
-    if ((e = cudaGetLastError())) return e;
+    cudaError_t e = cudaSuccess;
+    auto launch = [&](auto k, int warps, size_t sm) -> cudaError_t {
+        cudaError_t e2 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e2) return e2;
+        k<<<dim3(N, nfields), warps * 32, sm, st>>>(delta, K, tw_fwd, W, spill_on ? spill : nullptr);
+        return cudaGetLastError();
+    };
+    // FP32 planes that leave an SM one block take 16 warps instead of 8, for the latency of the rows' reads and of the
+    // transform's stages (64 fields of 256^3, K = 64: backward 19.56 -> 19.22 ms; one field 72 -> 68 us); where 8 warps
+    // fit twice, two blocks overlap each other's phases already
+    const size_t sm16 = plane_smem_n<T, N>(K, false, 16);
+    const bool wide = sizeof(T) == 4 && 2 * (sm8 + 1024) > 228 * 1024 && sm16 <= kMaxSmem;
+    if (spill_on) e = launch(fwd_plane_kernel<T, N, true, kPlaneWarps>, kPlaneWarps, plane_smem_n<T, N>(K, true));
+    else if (wide) {
+        if constexpr (sizeof(T) == 4) e = launch(fwd_plane_kernel<T, N, false, 16>, 16, sm16);
+    } else e = launch(fwd_plane_kernel<T, N, false, kPlaneWarps>, kPlaneWarps, sm8);
+    if (e) return e;
     const int nl = (2 * K + 1) * (K + 1);
     size_t smx = xlines_smem_n<T, N>();
     auto kx = fwd_xlines_kernel<T, N>;
