@@ -245,9 +245,6 @@ PS_DEV uint64_t mul2(uint64_t a, uint64_t b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-PS_DEV void lds2x2(uint32_t a, uint64_t& x, uint64_t& y) {  // 16 bytes of shared memory: two pairs
-    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "r"(a));
-}
 // hi = RN_bf16 pair of v; lo = RN_bf16 pair of the residuals v - hi, taken with one packed FP32
 // subtraction (exact: hi is within a factor 2 of each value).
 PS_DEV void split_pair(uint64_t v, uint32_t& hi, uint32_t& lo) {
