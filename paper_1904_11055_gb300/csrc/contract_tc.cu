@@ -463,6 +463,15 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
             tc::fence_proxy_async_smem();
             tc::tmem_st_wait();
             tc::fence_before_sync();
+            // At a window's last chunk, which this team drains, the window before must be over: this team may not have
+            // drained it, and where the window holds fewer chunks than there are slots its MMAs can still be running,
+            // when the wait for this window below would pass early.  The wait stands before this warp's arrival on
+            // produced[]: until then this window cannot complete, so acc_ready is in phase index - 1 or index and the
+            // parity is unambiguous (after the arrival it may already be in phase index + 1, which looks like index - 1
+            // and ends only with this warp's own drain).
+            win.advance_to(i, window);
+            const bool drains = i == win.end || i == nch - 1;
+            if (drains && win.index > 0 && !tc::mbar_wait_warp(acc_ready, (uint32_t)((win.index - 1) & 1), s_abort)) break;
             __syncwarp();
             if (lane == 0) {
                 tc::mbar_arrive(&empty[st]);
@@ -474,11 +483,7 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
                 ph_full ^= 1u;
             }
             // drain the accumulators after the last chunk of a window
-            win.advance_to(i, window);
-            if (i == win.end || i == nch - 1) {
-                // the window before must be over first: this team may not have drained it, and after a last window
-                // of fewer chunks than slots its MMAs can still be running, when the parity below would pass early
-                if (win.index > 0 && !tc::mbar_wait_warp(acc_ready, (uint32_t)((win.index - 1) & 1), s_abort)) break;
+            if (drains) {
                 if (!tc::mbar_wait_warp(acc_ready, (uint32_t)(win.index & 1), s_abort)) break;
                 tc::fence_after_sync();
                 for (int g = half; g < acc_cols / 16; g += 2) {
