@@ -143,6 +143,15 @@ int poly_diag_tc_tables(int N, int order, const double* edges, int nshell, unsig
                         int32_t* runs, int16_t* rowf, int16_t* colf, int32_t* binmap);
 
 /*
+ * The accumulation window of that contraction, in chunks of 32 cells: window
+ * (required) receives what a plan of these arguments would take, with the
+ * environment variable POLY_TC_WINDOW as it is set (a positive value replaces the
+ * default; values below the largest slot count, 4, are raised to it).  Returns a
+ * poly_status.
+ */
+int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsigned flags, int ell, int* window);
+
+/*
  * The adjoint's host tables (poly_backward), computed on the host alone.  The
  * gradient of B_b with respect to the field D_m at a cell is the sum, over the
  * positions of m in b, of the product of b's other fields there (Eq. estimator

@@ -1016,6 +1016,21 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
     return tc_build_layout(p, t, h, false, true, work);
 }
 
+// Accumulation window (chunks of 32 cells summed in FP32 in tensor memory before a drain).
+// The tensor-core FP32 accumulation error grows with the window; at 256^3 the largest
+// error over the split-BF16 scale is 1.3e-6 for the bispectrum at 128 chunks (6e-7 at 64;
+// the contraction takes 6.54 ms instead of 6.67), but 1.5e-5 for the trispectrum
+// (products of four fields) at 64 chunks, 5.9e-6 at 16.  The compact layouts take 14 (n = 4) and 12 (n = 5)
+// chunks, at which their error is that of the plain ones with 16.
+// POLY_TC_WINDOW sets another; one below the slot count is raised to it: a team that drains a window knows the
+// MMAs of the chunk that used its slot before to be complete, and with windows of at least as many chunks as slots
+// that chunk lies in the window or in the one before, so the wait for the one before cannot pass a phase early.
+static int tc_window(int order, int ra, int ca) {
+    const int def = order == 4 ? 14 : ra == 3 && ca == 2 ? 12 : order >= 5 ? 16 : 128;
+    const char* w = getenv("POLY_TC_WINDOW");
+    return w && atoi(w) > 0 ? std::max(atoi(w), kTcMaxSlots) : def;
+}
+
 // Launch shape of the contraction from the groups (host only): TMA stage bytes, B buffer
 // bytes, accumulator columns, A/B slot cap, shared memory and the producer team count.
 static poly_status tc_launch_shape(const PsPlan* p, const std::vector<TcGroup>& groups, TcState* t) {
@@ -1040,6 +1055,7 @@ static poly_status tc_launch_shape(const PsPlan* p, const std::vector<TcGroup>& 
     int min_slots = t->slot_cap;
     for (auto& g : groups) min_slots = std::min(min_slots, (512 - (g.acc_cols + 31) / 32 * 32) / (g.nmt * 32));
     t->teams = min_slots >= 3 ? 3 : 2;
+    t->window = tc_window(p->order, t->ra, t->ca);
     return POLY_OK;
 }
 
@@ -1081,15 +1097,6 @@ poly_status ps_tc_prepare(PsPlan* p) {
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return POLY_ERR_CUDA;
-    // Accumulation window (chunks of 32 cells summed in FP32 in tensor memory before a drain).
-    // The tensor-core FP32 accumulation error grows with the window; at 256^3 the largest
-    // error over the split-BF16 scale is 1.3e-6 for the bispectrum at 128 chunks (6e-7 at 64;
-    // the contraction takes 6.54 ms instead of 6.67), but 1.5e-5 for the trispectrum
-    // (products of four fields) at 64 chunks, 5.9e-6 at 16.  The compact layouts take 14 (n = 4) and 12 (n = 5)
-    // chunks, at which their error is that of the plain ones with 16.
-    t->window = p->order == 4 ? 14 : t->ra == 3 && t->ca == 2 ? 12 : p->order >= 5 ? 16 : 128;
-    const char* w = getenv("POLY_TC_WINDOW");
-    if (w && atoi(w) > 0) t->window = atoi(w);
     return POLY_OK;
 }
 
@@ -1153,6 +1160,24 @@ extern "C" int poly_diag_tc_tables(int N, int order, const double* edges, int ns
     try {
         return diag_tc_tables(N, order, edges, nshell, flags, ell, sms, max_mt, cta_mult, sizes, ctas, groups, mtiles,
                               runs, rowf, colf, binmap);
+    } catch (const std::bad_alloc&) {
+        return POLY_ERR_ALLOC;
+    }
+}
+
+extern "C" int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsigned flags, int ell, int* window) {
+    if (!window) return POLY_ERR_ARG;
+    try {
+        PsPlan hp;  // host tables only: no device call, no device memory
+        std::vector<short> lines;
+        if (poly_status s = ps_plan_host_tables(&hp, N, 1.0, order, nshell, edges, POLY_SPLIT_BF16, flags, ell, lines))
+            return s;
+        hp.sms = 152;  // sets the blocks, not the window
+        TcState t;
+        TcTables h;
+        if (poly_status s = tc_build_tables(&hp, &t, h)) return s;
+        *window = t.window;
+        return POLY_OK;
     } catch (const std::bad_alloc&) {
         return POLY_ERR_ALLOC;
     }

@@ -19,7 +19,7 @@ def test_short_last_windows(N, order, nshell, monkeypatch):
     e = fieldgen.unit_edges(nshell)
     d = torch.from_numpy(fieldgen.field("lognormal", N, 81, np.float32)).cuda()
     ref, scale = None, None
-    for window in (None, 5, 6, 7, 9, 11, 13, 16, 27, 64):
+    for window in (None, 1, 2, 3, 4, 5, 6, 7, 9, 11, 13, 16, 27, 64):
         if window is None:
             monkeypatch.delenv("POLY_TC_WINDOW", raising=False)
         else:

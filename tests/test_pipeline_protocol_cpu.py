@@ -17,11 +17,17 @@ issuer's MMAs complete phase w of `acc_ready` at the window's last chunk, the te
 the sums and completes phase w of `acc_free`, and the issuer starts window w + 1 only then.  Each warp
 of a team runs by itself between its arrival on `produced` and its drain.
 """
+import ctypes
 import os
 import random
 import re
 
+import numpy as np
 import pytest
+
+import fieldgen
+import paper_1904_11055_gb300 as ps
+from paper_1904_11055_gb300 import build as psbuild
 
 
 def run(T, S, nch, rng):
@@ -166,3 +172,24 @@ def test_waiting_after_the_arrival_can_stall():
     then asks for a phase whose parity the barrier will not show again."""
     rng = random.Random(5)
     assert "stall" in {run_drains(3, 3, 5, 21, False, rng) for _ in range(600)}
+
+
+@pytest.mark.parametrize("T,S,W", [(2, 4, 2), (2, 4, 1), (3, 3, 1), (3, 4, 1)])
+def test_windows_shorter_than_the_slots_can_go_wrong(T, S, W):
+    """The slot's previous chunk may then lie two or more windows back, and the wait for the window before passes early."""
+    rng = random.Random(10 * S + W)
+    assert any(run_drains(T, S, W, 8 * W + k % W, True, rng) is not None for k in range(2000))
+
+
+@pytest.mark.parametrize("order,nshell,default", [(3, 12, 128), (4, 10, 14), (2, 12, 128)])
+@pytest.mark.parametrize("env,window", [(None, None), ("1", 4), ("2", 4), ("3", 4), ("4", 4), ("5", 5), ("0", None)])
+def test_window_holds_at_least_as_many_chunks_as_slots(monkeypatch, order, nshell, default, env, window):
+    psbuild.build()
+    fn = ps.load_library().poly_diag_tc_window
+    fn.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_uint, ctypes.c_int, ctypes.c_void_p]
+    monkeypatch.delenv("POLY_TC_WINDOW", raising=False)
+    if env is not None:
+        monkeypatch.setenv("POLY_TC_WINDOW", env)
+    e, got = fieldgen.unit_edges(nshell), np.zeros(1, np.int32)
+    assert fn(64, order, e.ctypes.data, nshell, 0, 0, got.ctypes.data) == 0
+    assert got[0] == (window or default)
