@@ -146,10 +146,12 @@ int poly_diag_tc_tables(int N, int order, const double* edges, int nshell, unsig
  * The accumulation window of that contraction, in chunks of 32 cells: window
  * (required) receives what a plan of these arguments would take, with the
  * environment variable POLY_TC_WINDOW as it is set (a positive value replaces the
- * default; values below the largest slot count, 4, are raised to it).  Returns a
- * poly_status.
+ * default; values below 5, one more than the largest slot count, are raised to
+ * it); ends (NULL or int32 [nch]) the last chunk of each chunk's window in a
+ * block of nch chunks.  Returns a poly_status.
  */
-int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsigned flags, int ell, int* window);
+int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsigned flags, int ell, int nch,
+                        int* window, int32_t* ends);
 
 /*
  * The adjoint's host tables (poly_backward), computed on the host alone.  The

@@ -86,16 +86,29 @@ struct TcCta {  // one block: a group and a chunk range
     long long c0, c1;
 };
 
-// Window bookkeeping without divisions: the accumulators are drained after the
-// last chunk of each window of `window` chunks and after the block's last chunk.
+// Window bookkeeping without divisions in the loop: the accumulators are drained after the last chunk of each window.
+// All windows hold `window` chunks, but the first holds what is left.  (A short last window has no such order: the team
+// that drains it need not know that the window before, which another team drains, is over, and would have to wait for
+// that before it hands its last chunk on; every window's end waiting there cost the trispectrum of 256^3 / 32 shells
+// 2 %.)  A full window of more chunks than slots does know: the slot of its last chunk was used within the window, whose
+// MMAs start after the drain before.
 struct TcWindow {
     int end, index;  // last chunk of the current window, window number
-    __device__ TcWindow(int i0, int window) : end((i0 / window + 1) * window - 1), index(i0 / window) {}
-    __device__ void advance_to(int i, int window) {
+    __host__ __device__ TcWindow(int nch, int window) : end((nch - 1) % window), index(0) {}
+    __host__ __device__ void advance_to(int i, int window) {
         while (i > end) {
             end += window;
             index++;
         }
+    }
+    // the same for i = 0, 1, 2, ... in turn; true at a window's first chunk
+    __device__ bool next(int i, int window) {
+        const bool starts = i > end;
+        if (starts) {
+            end += window;
+            index++;
+        }
+        return starts || i == 0;
     }
 };
 
@@ -296,14 +309,13 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
             }
             // 64-bit descriptor = start address | LBO | (SBO, sm_100 descriptor version) << 32
             const uint64_t desc_k = ((uint64_t)((kSBO >> 4) | (1u << 14)) << 32) | (uint64_t)((kLBO >> 4) << 16);
-            TcWindow win(0, window);
+            TcWindow win(nch, window);
             int lst = 0;
             uint32_t lph = 0;  // stage and phase of empty[] that frees the stage for chunk c
             int slot = 0;
             uint32_t ph = 0;  // phase of produced[slot] for chunk i
             for (int i = 0; i < nch; i++) {
-                win.advance_to(i, window);
-                const bool wstart = i == win.end - window + 1;
+                const bool wstart = win.next(i, window);
                 if (!tc::mbar_wait_warp(&produced[slot], ph, s_abort)) break;
                 if (wstart && win.index > 0 && !tc::mbar_wait_warp(acc_free, (uint32_t)((win.index - 1) & 1), s_abort))
                     break;
@@ -329,7 +341,7 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
                         }
                     }
                     tc::mma_commit(&mma_done[slot]);
-                    if (i == win.end || i == nch - 1) tc::mma_commit(acc_ready);
+                    if (i == win.end) tc::mma_commit(acc_ready);
                 }
                 __syncwarp();
                 if (m == loader && c < nch) {
@@ -417,7 +429,7 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
         }
         int st = team;
         uint32_t ph_full = 0;
-        TcWindow win(team, window);
+        TcWindow win(nch, window);
         for (int i = team < nteams ? team : nch; i < nch; i += nteams) {
             if (!tc::mbar_wait_warp(&full[st], ph_full, s_abort)) break;
             const uint32_t D = sd0 + (uint32_t)(st * stage_bytes);
@@ -463,15 +475,6 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
             tc::fence_proxy_async_smem();
             tc::tmem_st_wait();
             tc::fence_before_sync();
-            // At a window's last chunk, which this team drains, the window before must be over: this team may not have
-            // drained it, and where the window holds fewer chunks than there are slots its MMAs can still be running,
-            // when the wait for this window below would pass early.  The wait stands before this warp's arrival on
-            // produced[]: until then this window cannot complete, so acc_ready is in phase index - 1 or index and the
-            // parity is unambiguous (after the arrival it may already be in phase index + 1, which looks like index - 1
-            // and ends only with this warp's own drain).
-            win.advance_to(i, window);
-            const bool drains = i == win.end || i == nch - 1;
-            if (drains && win.index > 0 && !tc::mbar_wait_warp(acc_ready, (uint32_t)((win.index - 1) & 1), s_abort)) break;
             __syncwarp();
             if (lane == 0) {
                 tc::mbar_arrive(&empty[st]);
@@ -483,7 +486,8 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
                 ph_full ^= 1u;
             }
             // drain the accumulators after the last chunk of a window
-            if (drains) {
+            win.advance_to(i, window);
+            if (i == win.end) {
                 if (!tc::mbar_wait_warp(acc_ready, (uint32_t)(win.index & 1), s_abort)) break;
                 tc::fence_after_sync();
                 for (int g = half; g < acc_cols / 16; g += 2) {
@@ -1022,13 +1026,11 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
 // the contraction takes 6.54 ms instead of 6.67), but 1.5e-5 for the trispectrum
 // (products of four fields) at 64 chunks, 5.9e-6 at 16.  The compact layouts take 14 (n = 4) and 12 (n = 5)
 // chunks, at which their error is that of the plain ones with 16.
-// POLY_TC_WINDOW sets another; one below the slot count is raised to it: a team that drains a window knows the
-// MMAs of the chunk that used its slot before to be complete, and with windows of at least as many chunks as slots
-// that chunk lies in the window or in the one before, so the wait for the one before cannot pass a phase early.
+// POLY_TC_WINDOW sets another, at least one chunk more than there are slots (TcWindow).
 static int tc_window(int order, int ra, int ca) {
     const int def = order == 4 ? 14 : ra == 3 && ca == 2 ? 12 : order >= 5 ? 16 : 128;
     const char* w = getenv("POLY_TC_WINDOW");
-    return w && atoi(w) > 0 ? std::max(atoi(w), kTcMaxSlots) : def;
+    return w && atoi(w) > 0 ? std::max(atoi(w), kTcMaxSlots + 1) : def;
 }
 
 // Launch shape of the contraction from the groups (host only): TMA stage bytes, B buffer
@@ -1165,8 +1167,9 @@ extern "C" int poly_diag_tc_tables(int N, int order, const double* edges, int ns
     }
 }
 
-extern "C" int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsigned flags, int ell, int* window) {
-    if (!window) return POLY_ERR_ARG;
+extern "C" int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsigned flags, int ell, int nch,
+                                   int* window, int32_t* ends) {
+    if (!window || nch < 0) return POLY_ERR_ARG;
     try {
         PsPlan hp;  // host tables only: no device call, no device memory
         std::vector<short> lines;
@@ -1177,6 +1180,11 @@ extern "C" int poly_diag_tc_window(int N, int order, const double* edges, int ns
         TcTables h;
         if (poly_status s = tc_build_tables(&hp, &t, h)) return s;
         *window = t.window;
+        TcWindow win(std::max(1, nch), t.window);
+        for (int i = 0; ends && i < nch; i++) {
+            win.advance_to(i, t.window);
+            ends[i] = win.end;
+        }
         return POLY_OK;
     } catch (const std::bad_alloc&) {
         return POLY_ERR_ALLOC;

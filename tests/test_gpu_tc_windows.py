@@ -1,8 +1,7 @@
-"""Accumulation windows of the tensor-core contraction whose last one is shorter than the A/B slots in flight: the
-team that drains it has not drained the window before, whose MMAs may still be running.  Windows that leave 1 to 4
-chunks to some blocks' last one, against the default window's result (its own test compares that with the
-oracle); a drain that came early would add a whole window twice (a relative error of one window in a block's
-chunks, 1e-2 and more here)."""
+"""Accumulation windows of the tensor-core contraction over window lengths that leave a block's short window 1 to 4
+chunks, and set lengths below the slot count (which are raised above it), against the default window's result (its own
+test compares that with the oracle); a drain that came early would add a whole window twice (a relative error of one
+window in a block's chunks, 1e-2 and more here)."""
 import numpy as np
 import pytest
 
@@ -15,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("N,order,nshell", [(64, 3, 16), (64, 4, 10), (48, 3, 12), (64, 2, 12)])
-def test_short_last_windows(N, order, nshell, monkeypatch):
+def test_short_windows(N, order, nshell, monkeypatch):
     e = fieldgen.unit_edges(nshell)
     d = torch.from_numpy(fieldgen.field("lognormal", N, 81, np.float32)).cuda()
     ref, scale = None, None

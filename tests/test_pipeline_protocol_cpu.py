@@ -12,10 +12,13 @@ The model explores random interleavings of the teams, the issuer and the MMA com
 checks that every wait starts with c in {u - 1, u} when T <= S (the rule the kernel enforces by
 capping its teams at its slots), and finds a schedule that breaks it when T > S.
 
-A second model covers the drains.  The accumulators are handed over once per window of W chunks: the
-issuer's MMAs complete phase w of `acc_ready` at the window's last chunk, the team of that chunk reads
-the sums and completes phase w of `acc_free`, and the issuer starts window w + 1 only then.  Each warp
-of a team runs by itself between its arrival on `produced` and its drain.
+A second model covers the drains.  The accumulators are handed over once per window of chunks: the
+issuer's MMAs complete phase w of `acc_ready` at the window's last chunk, the team of that chunk waits
+for it, reads the sums and completes phase w of `acc_free`, and the issuer starts window w + 1 only then.
+Each warp of a team runs by itself between its arrival on `produced` and its drain.  The wait is
+unambiguous where the team knows window w - 1 to be over, which the slot of the window's last chunk
+tells it when windows hold more chunks than there are slots; the kernel therefore gives the first
+window, not the last, the remainder.
 """
 import ctypes
 import os
@@ -87,21 +90,23 @@ def test_more_teams_than_slots_can_alias(T, S):
     assert any(run(T, S, 48, rng) is not None for _ in range(400))
 
 
-def run_drains(T, S, W, nch, early, rng, warps=2):
-    """One random schedule of the drains.  early: a warp waits for the window before its own arrival on `produced`
-    for a window's last chunk, else after it.  Returns None, or what went wrong: "stall" (no warp can move) or
-    the drain that read a window's sums before (or after) their time."""
-    nt = min(T, S)
-    last = lambda i: i == nch - 1 or i % W == W - 1
+def run_drains(T, S, ends, rng, wait=None, warps=2):
+    """One random schedule of the drains.  ends[i]: the last chunk of chunk i's window.  wait: None (each drain waits
+    for its own window alone), or "after" (a wait for the window before too, after the arrival on `produced`).
+    Returns None, or what went wrong: "stall" (no warp can move) or the drain that read a window's sums early."""
+    nch, nt = len(ends), min(T, S)
+    window = [0] * nch
+    for i in range(1, nch):
+        window[i] = window[i - 1] + (ends[i] != ends[i - 1])
     prog = []  # per warp: its steps in program order
     for t in range(nt):
         steps = []
         for i in range(t, nch, nt):
-            w = i // W
-            before = [("ready", w - 1)] if last(i) and w > 0 else []
-            steps += [("slot", i)] + (before if early else []) + [("arrive", i)]
-            if last(i):
-                steps += ([] if early else before) + [("ready", w), ("drain", w)]
+            w = window[i]
+            steps += [("slot", i), ("arrive", i)]
+            if i == ends[i]:
+                steps += [("ready", w - 1)] if wait == "after" and w > 0 else []
+                steps += [("ready", w), ("drain", w)]
         prog += [list(steps) for _ in range(warps)]
     pc = [0] * len(prog)
     arrived = [0] * nch
@@ -119,7 +124,7 @@ def run_drains(T, S, W, nch, early, rng, warps=2):
                 continue
             moves.append(k)
         can_issue = issued < nch and arrived[issued] == warps
-        if can_issue and issued % W == 0 and issued > 0 and free % 2 == (issued // W - 1) % 2:
+        if can_issue and issued and ends[issued] != ends[issued - 1] and free % 2 == (window[issued] - 1) % 2:
             can_issue = False
         if can_issue:
             moves.append("issue")
@@ -132,7 +137,7 @@ def run_drains(T, S, W, nch, early, rng, warps=2):
             issued += 1
         elif k == "complete":
             slot_phases[done % S] += 1
-            ready += last(done)
+            ready += done == ends[done]
             done += 1
         else:
             op, v = prog[k][pc[k]]
@@ -147,49 +152,46 @@ def run_drains(T, S, W, nch, early, rng, warps=2):
             pc[k] += 1
 
 
-def kernel_waits_before_arriving():
-    """Whether the contraction's producers wait for the window before ahead of their arrival on `produced`."""
-    path = os.path.join(os.path.dirname(__file__), "..", "paper_1904_11055_gb300", "csrc", "contract_tc.cu")
-    src = open(path).read()
-    body = src[src.index("// ------------------------------------------------------------- producers"):]
-    wait = re.search(r"mbar_wait_warp\(acc_ready, \(uint32_t\)\(\(win\.index - 1\) & 1\), s_abort\)", body)
-    return wait.start() < body.index("tc::mbar_arrive(&produced[slot]);")
+def last_window_short(nch, W):
+    return [min(nch - 1, i // W * W + W - 1) for i in range(nch)]
 
 
-DRAINS = [(2, 2, 5), (2, 3, 5), (2, 4, 4), (3, 3, 3), (3, 3, 7), (3, 4, 5), (3, 4, 4)]
-
-
-@pytest.mark.parametrize("T,S,W", DRAINS)
-def test_drains_neither_stall_nor_read_another_window(T, S, W):
-    rng = random.Random(100 * T + 10 * S + W)
-    early = kernel_waits_before_arriving()
-    for k in range(600):
-        assert run_drains(T, S, W, 3 * W + 1 + k % W, early, rng) is None
-
-
-def test_waiting_after_the_arrival_can_stall():
-    """Once every warp has arrived, the window may complete before a warp's wait for the one before starts: that wait
-    then asks for a phase whose parity the barrier will not show again."""
-    rng = random.Random(5)
-    assert "stall" in {run_drains(3, 3, 5, 21, False, rng) for _ in range(600)}
-
-
-@pytest.mark.parametrize("T,S,W", [(2, 4, 2), (3, 3, 1), (3, 4, 1)])
-def test_windows_shorter_than_the_slots_can_go_wrong(T, S, W):
-    """The slot's previous chunk may then lie two or more windows back, and the wait for the window before passes early."""
-    rng = random.Random(10 * S + W)
-    assert any(run_drains(T, S, W, 8 * W + k % W, True, rng) is not None for k in range(2000))
-
-
-@pytest.mark.parametrize("order,nshell,default", [(3, 12, 128), (4, 10, 14), (2, 12, 128)])
-@pytest.mark.parametrize("env,window", [(None, None), ("1", 4), ("2", 4), ("3", 4), ("4", 4), ("5", 5), ("0", None)])
-def test_window_holds_at_least_as_many_chunks_as_slots(monkeypatch, order, nshell, default, env, window):
+def kernel_windows(monkeypatch, order, nshell, nch, env):
+    """The window of a plan, and the last chunk of each chunk's window, from the library."""
     psbuild.build()
     fn = ps.load_library().poly_diag_tc_window
-    fn.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_uint, ctypes.c_int, ctypes.c_void_p]
+    fn.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_uint] + [ctypes.c_int] * 2 + \
+        [ctypes.c_void_p] * 2
     monkeypatch.delenv("POLY_TC_WINDOW", raising=False)
     if env is not None:
         monkeypatch.setenv("POLY_TC_WINDOW", env)
-    e, got = fieldgen.unit_edges(nshell), np.zeros(1, np.int32)
-    assert fn(64, order, e.ctypes.data, nshell, 0, 0, got.ctypes.data) == 0
-    assert got[0] == (window or default)
+    e, got, ends = fieldgen.unit_edges(nshell), np.zeros(1, np.int32), np.zeros(nch, np.int32)
+    assert fn(64, order, e.ctypes.data, nshell, 0, 0, nch, got.ctypes.data, ends.ctypes.data) == 0
+    return int(got[0]), ends.tolist()
+
+
+@pytest.mark.parametrize("T,S", [(2, 2), (2, 3), (2, 4), (3, 3), (3, 4)])
+@pytest.mark.parametrize("env", ["1", "2", "3", "4", "5", "6", "7"])
+def test_drains_neither_stall_nor_read_another_window(monkeypatch, T, S, env):
+    rng = random.Random(100 * T + 10 * S + int(env))
+    for nch in (1, 2, 3, 4, 5, 6, 13, 16, 17, 18, 19, 20):
+        _, ends = kernel_windows(monkeypatch, 3, 12, nch, env)
+        assert ends[-1] == nch - 1 and all(ends[i] >= i for i in range(nch))
+        for _ in range(60):
+            assert run_drains(T, S, ends, rng) is None
+
+
+@pytest.mark.parametrize("T,S,W,nch", [(2, 3, 5, 16), (3, 3, 5, 21), (3, 4, 5, 16)])
+def test_short_last_windows_go_wrong(T, S, W, nch):
+    """With the remainder in the last window its drain can come early; with a wait for the window before after the
+    arrival, that window may be over by two phases when the wait starts, whose parity then never shows again."""
+    rng = random.Random(10 * T + S)
+    ends = last_window_short(nch, W)
+    assert any("drain" in (run_drains(T, S, ends, rng) or "") for _ in range(2000))
+    assert any(run_drains(T, S, ends, rng, "after") == "stall" for _ in range(2000))
+
+
+@pytest.mark.parametrize("order,nshell,default", [(3, 12, 128), (4, 10, 14), (2, 12, 128)])
+@pytest.mark.parametrize("env,window", [(None, None), ("1", 5), ("3", 5), ("4", 5), ("5", 5), ("6", 6), ("0", None)])
+def test_window_holds_more_chunks_than_there_are_slots(monkeypatch, order, nshell, default, env, window):
+    assert kernel_windows(monkeypatch, order, nshell, 8, env)[0] == (window or default)
