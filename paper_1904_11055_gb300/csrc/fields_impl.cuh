@@ -508,13 +508,14 @@ static cudaError_t inverse_n(const Cx<T>* fhat, const short4* lines, const int* 
 // its own largest kz needs: shells whose plane buffer fits several times per SM
 // run as small blocks (SmallPlane), so that one block's transform phases overlap the
 // other's; the rest run as one 16-warp block per SM.  kz_host[s] is shell s's
-// largest kz (host array), kz_dev the same table on the device (or NULL).
+// largest kz (host array), kz_dev the same table on the device (or NULL); spill holds the planes
+// that do not fit shared memory (256^3 from K = 89 on; N ns blocks, else NULL).
 template <typename T, int N>
 static cudaError_t inverse_ranged_n(const Cx<T>* fhat, const short4* lines, const int* line_off, int s0, int ns, int K,
-                                    const Cx<double>* tw_inv, T* out, size_t out_stride, Cx<T>* xpre, int max_lines,
-                                    int tile_ns, const int* kz_host, const int* kz_dev, cudaStream_t st) {
+                                    const Cx<double>* tw_inv, T* out, size_t out_stride, Cx<T>* spill, Cx<T>* xpre,
+                                    int max_lines, int tile_ns, const int* kz_host, const int* kz_dev, cudaStream_t st) {
     if (plane_smem_n<T, N>(K, false, 16) > kMaxSmem || !xpre)
-        return inverse_n<T, N, false>(fhat, lines, line_off, s0, ns, K, 0, N, tw_inv, out, out_stride, nullptr, xpre,
+        return inverse_n<T, N, false>(fhat, lines, line_off, s0, ns, K, 0, N, tw_inv, out, out_stride, spill, xpre,
                                       max_lines, tile_ns, st);
     cudaError_t e;
     const size_t smx = xpass_smem_n<T, N>(K);

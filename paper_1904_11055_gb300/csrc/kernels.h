@@ -27,8 +27,8 @@ cudaError_t ps_inverse(int n, int is_double, int unity, const void* fhat, const 
 // kz (kz_host: host array indexed by shell; kz_dev: the same on the device, or
 // NULL); see inverse_ranged_n.
 cudaError_t ps_inverse_ranged_f32(int n, const void* fhat, const void* lines, const int* line_off, int s0, int ns, int K,
-                                  const void* tw_inv, void* out, size_t out_stride, void* xpre, int max_lines,
-                                  int tile_ns, const int* kz_host, const int* kz_dev, cudaStream_t st);
+                                  const void* tw_inv, void* out, size_t out_stride, void* spill, void* xpre,
+                                  int max_lines, int tile_ns, const int* kz_host, const int* kz_dev, cudaStream_t st);
 
 // ---- contract_cc.cu -----------------------------------------------------------
 // CUDA-core contraction: a task is a block of bins, one run of consecutive field

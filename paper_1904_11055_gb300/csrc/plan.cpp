@@ -736,8 +736,8 @@ poly_status ps_fields(PsPlan* p, const void* delta, cudaStream_t st) {
                        p->d_fields, (size_t)p->N * p->N * p->N, p->d_spill, p->d_xpre, p->max_lines, p->nfield, st);
     else
         e = ps_inverse_ranged_f32(p->N, p->d_fhat, p->d_lines, p->d_line_off, 0, p->nshell, p->K, p->d_tw_inv,
-                                  p->d_fields, (size_t)p->N * p->N * p->N, p->d_xpre, p->max_lines, p->nfield,
-                                  p->shell_kz.data(), p->d_shell_kz, st);
+                                  p->d_fields, (size_t)p->N * p->N * p->N, p->d_spill, p->d_xpre, p->max_lines,
+                                  p->nfield, p->shell_kz.data(), p->d_shell_kz, st);
     if (e) return cuda_error(e, "shell fields");
     p->launches += 2;  // x pass + plane kernel
     if (p->ell > 0) {
@@ -753,8 +753,8 @@ poly_status ps_fields(PsPlan* p, const void* delta, cudaStream_t st) {
                            p->nfield, st);
         else
             e = ps_inverse_ranged_f32(p->N, p->d_fhat_w, p->d_lines, p->d_line_off, 0, p->nshell, p->K, p->d_tw_inv,
-                                      out_w, (size_t)p->N * p->N * p->N, p->d_xpre, p->max_lines, p->nfield,
-                                      p->shell_kz.data(), p->d_shell_kz, st);
+                                      out_w, (size_t)p->N * p->N * p->N, p->d_spill, p->d_xpre, p->max_lines,
+                                      p->nfield, p->shell_kz.data(), p->d_shell_kz, st);
         if (e) return cuda_error(e, "weighted shell fields");
         p->launches += 3;
     }

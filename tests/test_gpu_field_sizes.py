@@ -40,3 +40,37 @@ def test_fields_match_the_transform_of_the_masked_spectrum(N, prec):
         ref = (torch.fft.ifftn(F * shell_mask(q2, edges, s)).real * N**3).cpu().numpy()
         err = np.abs(got[s] - ref).max() / np.abs(ref).max()
         assert err < tol, (s, err, tol)
+
+
+@pytest.mark.parametrize("prec,ell", [("fp32", 0), ("split_bf16", 0), ("split_bf16", 2)])
+@pytest.mark.parametrize("K", [88, 89, 120])
+def test_planes_beyond_shared_memory(K, prec, ell):
+    """Single-precision planes of 256^3 fit shared memory up to K = 88; from 89 on they go through a buffer.  The
+    fields as above, the power spectrum against the mean of |delta_hat|^2, and the gradient by Euler's theorem,
+    delta . dB = 2 B.  Bounds: FP32 sums of squares over 512 cells, then FP64, 1e-5; split-BF16, the tensor core
+    truncates a growing sum at each of a window's 128 x 2 x 3 accumulations by up to 2^-24 of it."""
+    N, edges = 256, np.array([1.0, 30.5, K - 4.5, K + 0.5])
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    d = torch.randn(N, N, N, generator=gen, device="cuda", dtype=torch.float32)
+    plan = ps.Plan(N, 100.0, 2, edges, prec, 0, ell)
+    B = plan.estimate(d)
+    plan.sync()
+    F = torch.fft.fftn(d.double())
+    f, q2 = grid_q2(N)
+    w = (2 * ell + 1) * (1.5 * f[None, None, :] ** 2 / q2.clamp(min=1.0) - 0.5) if ell else torch.ones_like(q2)
+    P = (F.abs() ** 2 * w, F.abs() ** 2 * w.abs())
+    c = 100.0**3 / float(N) ** 6
+    tol = 768 * 2.0**-24 if prec == "split_bf16" else 1e-5
+    for s in range(3):
+        m = shell_mask(q2, edges, s)
+        assert abs(float(B[s]) - c * float(P[0][m].mean())) <= tol * c * float(P[1][m].mean())
+    if ell:
+        return
+    got = library_fields(plan, d)
+    for s in range(3):
+        ref = (torch.fft.ifftn(F * shell_mask(q2, edges, s)).real * N**3).cpu().numpy()
+        assert np.abs(got[s] - ref).max() / np.abs(ref).max() < 8 * math.log2(N**3) * 2.0**-24
+    wt = torch.tensor([1.0, 0.5, 2.0], dtype=torch.float64, device="cuda")
+    g = plan.backward(d, wt)
+    plan.sync()
+    assert float((g.double() * d.double()).sum()) == pytest.approx(2 * float((wt * B).sum()), rel=2 * tol)
