@@ -23,8 +23,9 @@
 //
 // Fields of one block's tasks arrive by 16-byte asynchronous copies of every thread
 // (stages of a few chunks) and serve its 12 warps; one bulk copy per run of fields
-// and chunk, about a KB each, took 58 ms.  FP32 lane sums cover 256 steps; then they
-// are summed over the warp and added to FP64 sums.  FP64 throughout for the plain
+// and chunk, about a KB each, took 58 ms.  FP32 lane sums cover 256 steps (two
+// sums, of the even and the odd cells); then they are added over the warp with their rounding errors and go to FP64
+// sums.  FP64 throughout for the plain
 // method and the exact polygon counts over the symmetry wedge (cell weights on the
 // rows).
 #include <algorithm>
@@ -72,7 +73,8 @@ struct CcLane<float> {
         return c;
     }
     static PS_DEV V abs(V a) { return a & 0x7fffffff7fffffffull; }
-    static PS_DEV float sum(V a) { return __uint_as_float((uint32_t)a) + __uint_as_float((uint32_t)(a >> 32)); }
+    static PS_DEV float lo(V a) { return __uint_as_float((uint32_t)a); }
+    static PS_DEV float hi(V a) { return __uint_as_float((uint32_t)(a >> 32)); }
 };
 template <>
 struct CcLane<double> {
@@ -88,7 +90,6 @@ struct CcLane<double> {
     static PS_DEV V mul(V a, V b) { return a * b; }
     static PS_DEV V mad(V a, V b, V c) { return fma(a, b, c); }
     static PS_DEV V abs(V a) { return fabs(a); }
-    static PS_DEV double sum(V a) { return a; }
 };
 
 // The products of one value per leg of legs [L0, L1), the first leg's index slowest; leg l's values at d[S::at(l)].
@@ -108,26 +109,40 @@ PS_DEV void cc_products(const typename CcLane<T>::V* d, typename CcLane<T>::V* o
     }
 }
 
+// a + b: the rounded sum, and in e its rounding error (Knuth's two-sum; not a number where the sum is infinite).
+PS_DEV float cc_two_sum(float a, float b, float& e) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+    return s;
+}
+
 // Sum of V values over the warp's 32 lanes by halving: after the exchange at lane distance d a
 // lane keeps the half of the values that its bit d selects.  V = 64: lane l ends with values
-// 2 l' and 2 l' + 1, l' = the bits of l (16 first) as the high bits of the value index.
+// 2 l' and 2 l' + 1, l' = the bits of l (16 first) as the high bits of the value index.  FP32
+// values carry their sum's rounding error beside them (e), so that what FP64 takes over is the
+// lanes' sums added to about 48 bits; adding them in FP64 costs 8 % (256^3 / 64 shells 37.3 and 40.7 ms).
 template <typename T, int V>
-PS_DEV void cc_warp_sum(T* v, int lane) {
+PS_DEV void cc_warp_sum(T* v, T* e, int lane) {
     int n = V;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
-        const bool up = lane & d;
-        if (n > 1) {
-            n >>= 1;
+        const bool halve = n > 1, up = halve && (lane & d);
+        if (halve) n >>= 1;
 #pragma unroll
-            for (int i = 0; i < V / 2; i++)
-                if (i < n) {
-                    const T keep = up ? v[i + n] : v[i], give = up ? v[i] : v[i + n];
-                    v[i] = keep + __shfl_xor_sync(0xffffffffu, give, d);
+        for (int i = 0; i < V / 2; i++)
+            if (i < n) {
+                const int k = halve ? i + n : i;
+                const T keep = up ? v[k] : v[i], give = up ? v[i] : v[k];
+                const T other = __shfl_xor_sync(0xffffffffu, give, d);
+                if constexpr (sizeof(T) == 4) {
+                    const T ekeep = up ? e[k] : e[i], egive = up ? e[i] : e[k];
+                    T err;
+                    v[i] = cc_two_sum(keep, other, err);
+                    e[i] = ekeep + __shfl_xor_sync(0xffffffffu, egive, d) + err;
+                } else {
+                    v[i] = keep + other;
                 }
-        } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
-        }
+            }
     }
 }
 
@@ -191,17 +206,23 @@ __global__ void __launch_bounds__(kCcThreads, 1)
     for (int i = 0; i < (V + 31) / 32; i++) acc64[i] = 0.0;
 
     auto flush = [&]() {
-        T v[V];
+        constexpr int E = sizeof(T) == 4 ? V : 1;
+        T v[V], e[E];
 #pragma unroll
         for (int i = 0; i < S::rows; i++)
 #pragma unroll
             for (int j = 0; j < S::cols; j++) {
-                v[i * S::cols + j] = Ln::sum(acc[i][j]);
+                const int k = i * S::cols + j;
+                if constexpr (sizeof(T) == 4) v[k] = cc_two_sum(Ln::lo(acc[i][j]), Ln::hi(acc[i][j]), e[k]);
+                else v[k] = acc[i][j];
                 acc[i][j] = Ln::zero();
             }
-        cc_warp_sum<T, V>(v, lane);
+        cc_warp_sum<T, V>(v, e, lane);
 #pragma unroll
-        for (int i = 0; i < (V + 31) / 32; i++) acc64[i] += (double)v[i];
+        for (int i = 0; i < (V + 31) / 32; i++) {
+            acc64[i] += (double)v[i];
+            if constexpr (sizeof(T) == 4) acc64[i] += e[i] == e[i] ? (double)e[i] : 0.0;  // an infinite sum has no error term
+        }
     };
 
     const uint32_t p0 = smem + Ln::offset(lane, chunk_bytes);

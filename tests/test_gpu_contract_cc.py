@@ -35,3 +35,19 @@ def test_blocks_match_oracle(prec, N, order, nshell, flags):
     assert np.max(np.abs(B - ref["B"])[some] / (c * ref["scale"][some])) <= TOL[prec]
     assert np.max(np.abs(scale - ref["scale"])[some] / ref["scale"][some]) <= TOL[prec]
     plan.close()
+
+
+def test_fp32_lanes_are_added_without_rounding():
+    """FP32 sums are rounded within a lane only (some hundred cells).  Three waves of a quarter of the grid's frequency
+    with 11-bit amplitudes make every cell's square an integer of at most 23 bits times a power of two, which a lane's
+    few cells of this plan add without rounding; the lanes' sums together take 30 bits and more."""
+    N, L = 64, 500.0
+    c = torch.cos(0.5 * np.pi * torch.arange(N, dtype=torch.float64)).round()
+    d = 947 * c[:, None, None] + 613 * c[None, :, None] + 311 * c[None, None, :]
+    plan = ps.Plan(N, L, 2, np.array([15.5, 16.5]), "fp32")
+    B, scale = plan.estimate(d.float().cuda(), scale=True)
+    S = float((d ** 2).sum())  # sum of D^2 over N^6, an integer below 2^53
+    want = L ** 3 * S / (float(N) ** 3 * float(plan.counts[0]))
+    assert float(B[0]) == pytest.approx(want, rel=1e-12)
+    assert float(scale[0]) * L ** 3 / float(N) ** 6 == pytest.approx(want, rel=1e-12)
+    plan.close()
