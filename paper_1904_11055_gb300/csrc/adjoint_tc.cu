@@ -290,19 +290,18 @@ __global__ void __launch_bounds__(kAtThreads, 1)
 // The same gradient as one GEMM over pairs of shells, for up to 64 shells:
 //   G_m(x) = sum_p P_p(x) W[p][m],  P_p = D_i D_j of the pair p = (i <= j).
 // M = 128 cells (TMEM lanes), K = the pairs, N = the shells m.  The products are formed in FP32, split into
-// bf16 hi + lo and written to TMEM (A); the weights (B, hi and lo) stream through shared memory.
+// bf16 hi + lo and written to TMEM (A); the weights (B), split into three bf16 parts, stream through shared memory.
 //
 // Why: T[x][(m, j)] = sum_i W_m[i][j] D_i (above) multiplies every cell with 3,584 columns x 64 shells and
 // reduces the columns on the CUDA cores; the pairs need 2,304 products a cell, 64 columns, no reduction, and
 // skip the columns that a pair's triangles do not reach (at 64 shells a quarter of them).  256^3 / 64 shells:
-// 26.2 -> 13.9 ms (10.4 without what the precision asks for, below).  What bounds it: the producers' instructions
-// (seven per two products and as many around them) and the barriers of each chunk; without the lo x lo products
-// 62 % of the issue slots, the ALU pipe of the bf16 conversions 48 % busy, the tensor pipe 37 %.
+// gradient 31.9 -> 18.3 ms.  What bounds it: the producers' instructions (seven per two products and as many around
+// them) and the barriers of each chunk.
 //
 // K comes in chunks of 64 pairs: 8 consecutive i by 8 consecutive j, so that a lane keeps its 8 D_j in
 // registers over a run of chunks and loads 8 values per 64 products.  (Chunks of 32 pairs ran 12.6 ms instead of
-// 10.4 at 256^3 / 64 shells, 10 ms of it without the products and two thirds of the MMAs: the barriers around a
-// chunk set the pace.)  A chunk's columns are the 16-column blocks that hold one of its weights (the first chunk
+// 10.4 at 256^3 / 64 shells in a first form, 10 ms of it without the products and two thirds of the MMAs: the barriers
+// around a chunk set the pace.)  A chunk's columns are the 16-column blocks that hold one of its weights (the first chunk
 // of a segment takes them all and overwrites, which starts the sums).  The weights of absent entries are zero.
 //
 // A block takes tiles of 256 cells (two M tiles).  12 producer warps in three groups: group g forms both M
@@ -311,9 +310,16 @@ __global__ void __launch_bounds__(kAtThreads, 1)
 // M tile, one warp for the copies: the tile's fields (one bulk copy, two buffers) and the chunks' weights (a
 // ring).  The accumulators are summed over segments of a few chunks only, because the tensor core's FP32
 // accumulation truncates (relative 2^-25 per MMA): the producer warps add a finished segment to their FP32 sums
-// (rounded to nearest).  The lo x lo products are added too (the tensor pipe has the room), and up to 32 shells
-// the cross products have sums of their own, so that fewer additions truncate the large ones: the error against
-// 64 bits is then no larger than that of the columns (m, j).
+// (rounded to nearest).
+//
+// Precision.  The error against 64 bits must not be above that of the columns (m, j).  Four products of parts are
+// added, P hi x W0, P hi x W1, P lo x W0 and P hi x W2; the third part of the weights takes their rounding (2^-17 of
+// each) out and costs 1 % of the time.  (P lo x W1 in place of P hi x W2: 2.7e-6 to 2.9e-6 with normal weights in these
+// orders, up to 3 % above the columns'; both: 1.06 times the time.)  Two orders keep what is truncated small:
+// the small products of a chunk come before its hi x W0, and the chunks of large shells, where a field's power falls
+// with k, before those of small ones; up to 32 shells the small products have sums of their own.  Normal weights,
+// 256^3 / 64 shells: columns 2.88e-6, pairs 4.8e-7; 128^3 / 20 shells 2.83e-6 and 3.8e-7; weights over the bins'
+// expected scatter below.
 constexpr int kAqCells = 256;    // cells of a tile
 constexpr int kAqMaxShells = 64;
 constexpr int kAqProd = 12;      // producer warps
@@ -321,31 +327,42 @@ constexpr int kAqThreads = 32 * (kAqProd + 3);
 constexpr int kAqGroups = 3;     // groups of four producer warps
 constexpr int kAqSlots = 3;      // A slots (>= kAqGroups), each both M tiles' products of one chunk
 constexpr int kAqRing = 4;       // chunks of weights in shared memory
-// chunks per accumulation segment (16 accumulations each; 3 at 33-48 shells), above 32 shells: 256^3 / 64 shells
-// 20.7 ms a gradient with 6 (error 3.4e-6 against 64 bits), 21.1 with 5 (3.2e-6), 21.6 with 4 (3.1e-6)
-constexpr int kAqSeg = 4;
-constexpr int kAqSegSplit = 12;  // with the cross products in sums of their own (48), up to 32 shells
+// Chunks per accumulation segment (16 accumulations each), above 32 shells.  Weights over the bins' expected scatter, so
+// that all chunks count alike; error of the columns, then of the pairs with 3, 4, 6 and 12 chunks, in 1e-6, and ms a gradient:
+//   256^3 / 64 shells  2.89   1.74 1.91 2.26 3.66   20.0 19.1 18.3 16.9
+//   256^3 / 52 shells  2.72   1.40 1.60 1.83 2.56   15.0 14.2 13.8 12.9
+//   128^3 / 40 shells  3.20   2.29 2.35 2.60 2.95   1.48 1.44 1.41 1.36
+// With 6: 128^3 / 60 shells of width 0.7 3.28 and 2.72, 256^3 / 57 of width 1.4 3.24 and 2.59, 160^3 / 48 3.19 and 2.36.
+constexpr int kAqSeg = 6;
+// With the small products in sums of their own (4 large accumulations a chunk), up to 32 shells: 128^3 / 32 shells 2.92
+// for the columns, 1.58 with 6 chunks at 0.985 ms, 1.68 with 12 at 0.943.
+constexpr int kAqSegSplit = 12;
+static_assert(kAqSegSplit >= kAqGroups, "chunks added without products must share their segment with one that has some");
 constexpr int kAqDelay = kAqGroups;      // chunks after a segment's end at which a group reads its sums: one chunk of each group
 constexpr int kAqBar = 64;       // mbarriers and flags, in 8-byte words
 
 struct AqChunk {
     int jb, i0;      // first j, first i (8 of each); jb < 0: no products (nn = 0)
     int n0, nn;      // columns [n0, n0 + nn)
-    int b_off;       // byte offset of its weights (hi, then lo: nn * 128 bytes each)
+    int b_off;       // byte offset of its weights (three parts of nn * 128 bytes)
     int first, last; // first / last chunk of its segment
     int end;         // entry s: last chunk of the tile's segment s
 };
 
-// weights to their places: hi at place, lo lo_off bytes after it
+constexpr int kAqBCol = 3 * 128;  // bytes of a chunk's weights per column: 64 pairs, three parts
+
+// weights to their places: the parts at place.x, place.y bytes apart
 __global__ void aq_scatter_kernel(const float* __restrict__ w, const int2* __restrict__ place, int nent,
                                   uint8_t* __restrict__ b) {
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nent; e += gridDim.x * blockDim.x) {
         const int2 p = place[e];
-        const float v = w[e];
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-        *reinterpret_cast<uint16_t*>(b + p.x) = *reinterpret_cast<const uint16_t*>(&h);
-        *reinterpret_cast<uint16_t*>(b + p.x + p.y) = *reinterpret_cast<const uint16_t*>(&l);
+        float v = w[e];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const __nv_bfloat16 h = __float2bfloat16_rn(v);
+            *reinterpret_cast<uint16_t*>(b + p.x + k * p.y) = *reinterpret_cast<const uint16_t*>(&h);
+            v -= __bfloat162float(h);  // exact
+        }
     }
 }
 
@@ -401,7 +418,7 @@ __global__ void __launch_bounds__(kAqThreads, 1)
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *s_tmem;
-    // accumulators of M tile t at column 64 t, up to 32 shells the cross products' 32 columns on; A slot s of M tile t at 128 + 128 s + 64 t
+    // accumulators of M tile t at column 64 t, up to 32 shells the small products' 32 columns on; A slot s of M tile t at 128 + 128 s + 64 t
     const int ntl = ((int)blockIdx.x < ntile) ? (ntile - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const uint32_t cross = nblk16 <= 2 ? 32u : 0u;
     const int total = ntl * nchunk;  // chunks this block runs (a tile's chunks in a row, tile after tile)
@@ -430,9 +447,9 @@ __global__ void __launch_bounds__(kAqThreads, 1)
                 }
                 if (cg >= kAqRing && !tc::mbar_wait(b_free + rs, rph, s_abort)) break;
                 const AqChunk ch = s_ch[c];
-                tc::mbar_arrive_expect_tx(b_full + rs, (uint32_t)(ch.nn * 256));
+                tc::mbar_arrive_expect_tx(b_full + rs, (uint32_t)(ch.nn * kAqBCol));
                 if (ch.nn > 0)
-                    tc::bulk_load(s_b + (size_t)rs * b_stage, b_g + ch.b_off, (uint32_t)(ch.nn * 256), b_full + rs);
+                    tc::bulk_load(s_b + (size_t)rs * b_stage, b_g + ch.b_off, (uint32_t)(ch.nn * kAqBCol), b_full + rs);
                 b_iss = cg + 1;
                 if (++rs == kAqRing) {
                     rs = 0;
@@ -470,18 +487,22 @@ __global__ void __launch_bounds__(kAqThreads, 1)
             if (el) {
                 const uint32_t d = tmem + (uint32_t)(64 * t + ch.n0);
                 const uint32_t a = tmem + 128u + (uint32_t)(128 * slot + 64 * t);
-                const uint32_t bh = tc::smem_u32(s_b + (size_t)rs * b_stage), bl = bh + (uint32_t)(ch.nn * 128);
+                const uint32_t b0 = tc::smem_u32(s_b + (size_t)rs * b_stage), part = (uint32_t)(ch.nn * 128);
                 const uint32_t idesc = tc::idesc_bf16(128, ch.nn);
-                const uint32_t dx = d + cross, fx = ch.first && cross ? 0u : 1u;
+                const uint32_t dx = d + cross;
+                if (ch.nn > 0) {
+                    auto desc = [&](uint32_t b) { return desc_k | (uint64_t)((b >> 4) & 0x3FFFu); };
 #pragma unroll
-                for (int ks = 0; ks < 4 && ch.nn > 0; ks++) {
-                    const uint64_t dh = desc_k | (uint64_t)(((bh + ks * 256) >> 4) & 0x3FFFu);
-                    const uint64_t dl = desc_k | (uint64_t)(((bl + ks * 256) >> 4) & 0x3FFFu);
-                    const uint32_t ah = a + (uint32_t)(8 * ks), al = ah + 32u;
-                    tc::mma_ts(d, ah, dh, idesc, ks == 0 && ch.first ? 0u : 1u);  // hi x hi
-                    tc::mma_ts(dx, ah, dl, idesc, ks == 0 ? fx : 1u);             // hi x lo
-                    tc::mma_ts(dx, al, dh, idesc, 1u);                            // lo x hi
-                    tc::mma_ts(dx, al, dl, idesc, 1u);                            // lo x lo
+                    for (int ks = 0; ks < 4; ks++) {
+                        const uint32_t ah = a + (uint32_t)(8 * ks), al = ah + 32u, b = b0 + (uint32_t)(256 * ks);
+                        tc::mma_ts(dx, ah, desc(b + 2 * part), idesc, ks == 0 && ch.first ? 0u : 1u);  // hi x W2
+                        tc::mma_ts(dx, ah, desc(b + part), idesc, 1u);                                 // hi x W1
+                        tc::mma_ts(dx, al, desc(b), idesc, 1u);                                        // lo x W0
+                    }
+#pragma unroll
+                    for (int ks = 0; ks < 4; ks++)  // hi x W0
+                        tc::mma_ts(d, a + (uint32_t)(8 * ks), desc(b0 + (uint32_t)(256 * ks)), idesc,
+                                   ks == 0 && ch.first && cross ? 0u : 1u);
                 }
                 tc::mma_commit(freed + slot);
                 tc::mma_commit(b_free + rs);
@@ -746,6 +767,7 @@ static poly_status at_build_tables(const PsPlan* p, const std::vector<int>& ent_
     }
     S->nent = (int)ent.size();
     // at least half the SM's shared memory: one block per SM, so no block waits in tcgen05.alloc for another
+    // (64 shells: 231,040 bytes of the 232,448 a block may have)
     S->smem = std::max<size_t>(at_smem_bytes(S->max_nchunk, S->max_nchunk, kp), 116 * 1024);
     const int64_t ntile = (ncell + kAtCells - 1) / kAtCells;
     const int npairs = ((int)S->groups.size() + 1) / 2;
@@ -768,13 +790,14 @@ static void aq_build_tables(const PsPlan* p, const std::vector<int>& ent_m, cons
     if (cols.empty()) cols[{0, 0}] = {0, 0};  // no entry at all: one chunk of zeros
     S->nblk16 = (p->nshell + 15) / 16;
     // every group takes part in every tile (it is what frees the tile's fields): at least kAqGroups chunks, the
-    // added ones without products
-    const int n = std::max<int>((int)cols.size(), kAqGroups), per = S->nblk16 <= 2 ? kAqSegSplit : S->nblk16 == 3 ? kAqSeg - 1 : kAqSeg;
+    // added ones without products (up to 16 shells only, so in the last chunk's segment)
+    const int n = std::max<int>((int)cols.size(), kAqGroups), per = S->nblk16 <= 2 ? kAqSegSplit : kAqSeg;
     const int nseg = (n + per - 1) / per;
     std::map<std::pair<int, int>, int> at;
     b_total = 0;
     int k = 0, seg = 0;
-    for (auto& kv : cols) {  // j blocks ascending, i ascending within
+    for (auto it = cols.rbegin(); it != cols.rend(); ++it) {  // j blocks descending, i descending within
+        const auto& kv = *it;
         AqChunk c{};
         c.jb = 8 * kv.first.first;
         c.i0 = 8 * kv.first.second;
@@ -783,7 +806,7 @@ static void aq_build_tables(const PsPlan* p, const std::vector<int>& ent_m, cons
         c.n0 = c.first ? 0 : 16 * kv.second.first;
         c.nn = c.first ? 16 * S->nblk16 : 16 * (kv.second.second + 1 - kv.second.first);
         c.b_off = (int)b_total;
-        b_total += (size_t)c.nn * 256;
+        b_total += (size_t)c.nn * kAqBCol;
         at[kv.first] = k++;
         seg += c.last;
         S->chunks.push_back(c);
@@ -805,7 +828,8 @@ static void aq_build_tables(const PsPlan* p, const std::vector<int>& ent_m, cons
     }
     S->nent = (int)ent.size();
     // at least half the SM's shared memory: one block per SM, so no block waits in tcgen05.alloc for another
-    S->smem = std::max<size_t>(2 * (size_t)kAqCells * p->nshell * 4 + (size_t)kAqRing * S->nblk16 * 16 * 256 +
+    // (64 shells: 231,040 bytes of the 232,448 a block may have)
+    S->smem = std::max<size_t>(2 * (size_t)kAqCells * p->nshell * 4 + (size_t)kAqRing * S->nblk16 * 16 * kAqBCol +
                                    S->chunks.size() * sizeof(AqChunk) + kAqBar * 8,
                                116 * 1024);
     S->pairs = true;
@@ -936,7 +960,7 @@ cudaError_t ps_at_contract(PsPlan* p, AtState* S, const float* w, cudaStream_t s
         const int ntile = (int)(ncell / kAqCells);  // N^3 is a multiple of 256
         at_pairs_kernel<<<std::min(p->sms, ntile), kAqThreads, S->smem, st>>>(
             (const float*)p->d_fields, p->nshell, ncell, ntile, (const AqChunk*)S->d_chunks, (int)S->chunks.size(), S->nblk16,
-            (const uint8_t*)S->d_b, S->nblk16 * 16 * 256, (float*)p->d_G, S->d_err);
+            (const uint8_t*)S->d_b, S->nblk16 * 16 * kAqBCol, (float*)p->d_G, S->d_err);
         return cudaGetLastError();
     }
     at_scatter_kernel<<<nb, 256, 0, st>>>(w, (const int*)S->d_pos, S->nent, (uint16_t*)S->d_bhi, (uint16_t*)S->d_blo);

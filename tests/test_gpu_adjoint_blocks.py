@@ -43,3 +43,26 @@ def test_pair_gradient_matches_oracle(N, nshell, width):
     (48, 4, 9, "fp64", 0), (32, 3, 9, "fp64", ps.POLY_BINS_ALL_SORTED)])
 def test_gradient_blocks_match_oracle(N, order, nshell, prec, flags):
     check(N, order, fieldgen.unit_edges(nshell), prec, flags, 70 + nshell)
+
+
+@pytest.mark.parametrize("nshell", [20, 40, 52, 64])
+def test_pair_gradient_error_against_64_bits(nshell):
+    """The pairs' errors stay below those of the form over columns (m, j), which is what runs beyond 64 shells (2.8e-6 of
+    the 2-norm with normal weights, 2.6e-6 to 3.2e-6 with weights over the bins' expected scatter).  Bounds: products
+    split into bf16 hi + lo leave 2^-18 of each on average at random, below 5e-7 of the sum; then the tensor core's
+    truncation, 2^-25 of the running sum for each of a segment's 96 accumulations, 2.9e-6 if all of them fell on the
+    full sum.  With normal weights the last chunk holds nearly all of the sum, and 16 accumulations, 4.8e-7."""
+    N = 128 if nshell <= 40 else 256
+    e = fieldgen.unit_edges(nshell)
+    x = torch.from_numpy(fieldgen.field("lognormal", N, 6, np.float32)).cuda()
+    p64, p = ps.Plan(N, 500.0, 3, e, "fp64"), ps.Plan(N, 500.0, 3, e, "split_bf16")
+    k = p.bins.astype(np.float64)
+    scatter = np.exp(0.5 * (2.5 * np.log(k) + (k / (N / 4)) ** 2)).prod(axis=1)
+    for seed in (1, 2, 4):
+        r = np.random.default_rng(seed).standard_normal(p.nbins) * (p.counts > 0)
+        for w, bound in ((r, 1e-6), (r * scatter, 3.4e-6)):
+            w = torch.from_numpy(w).cuda()
+            ref, g = p64.backward(x.double(), w), p.backward(x, w)
+            p64.sync(), p.sync()
+            assert float((g.double() - ref).norm() / ref.norm()) <= bound
+    p64.close(), p.close()
