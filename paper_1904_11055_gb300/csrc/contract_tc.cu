@@ -433,9 +433,8 @@ __global__ void __launch_bounds__(tc_threads(TEAMS), 1)
         for (int i = team < nteams ? team : nch; i < nch; i += nteams) {
             if (!tc::mbar_wait_warp(&full[st], ph_full, s_abort)) break;
             const uint32_t D = sd0 + (uint32_t)(st * stage_bytes);
-            // two teams: the first tile's products before the wait for the slot, which they then cover (two
-            // teams, three slots: trispectrum 256^3 / 32 shells 12.95 -> 12.66 ms; three teams cover each other's
-            // waits and have no registers for it)
+            // two teams: the first tile's products before the wait for the slot, which they then cover; three teams
+            // cover each other's waits and have no registers for it
             uint32_t v0[16];
             if (TEAMS == 2) tc_row_products<RA>(D + key1[0], D + key2[0], RA == 3 ? D + key3[0] : 0u, v0);
             const int slot = i % nslots, use = i / nslots;  // slot and its use count
@@ -1000,18 +999,21 @@ static poly_status tc_build_layout(const PsPlan* p, TcState* t, TcTables& h, boo
     return tc_launch_shape(p, h.groups, t);
 }
 
-// The plain layout, and for orders 4 and 5 the compact one where it is no more work.  What the plain layout
-// refuses stays refused, so the plans taken do not depend on the layout.  Contraction, plain -> compact: n = 4,
-// 256^3 / 32 shells 21.4 -> 13.2 ms, 160^3 / 26 3.11 -> 1.68, 128^3 / 20 0.76 -> 0.71, 64^3 / 8 the same; n = 5,
-// 128^3 / 20 shells 4.96 -> 2.1.  Plans of order 5 up to 16 shells keep the plain layout, which the
+// The plain layout, and for orders 4 and 5 the compact one where it is no more work; two producer teams take 1.15 times
+// as long as three (1.05 to 1.14 measured on one layout).  What the plain layout
+// refuses stays refused, so the plans taken do not depend on the layout.  Estimates, plain -> compact in ms: n = 4,
+// 256^3 / 32 shells 21.6 -> 13.5, 28 (three teams, two) 16.2 -> 15.7, 34 (the same) 25.8 -> 22.2, but 33 (the same)
+// 21.2 -> 22.3: not taken; 27 the same work, 160^3 / 26 3.5 -> 2.0, 128^3 / 20 0.91 -> 0.86, 64^3 / 10 the same; n = 5,
+// 128^3 / 20 shells 5.1 -> 2.3.  Plans of order 5 up to 16 shells keep the plain layout, which the
 // host-table tests hold them to (not measured there in the compact one).
 static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
     double work = 0, cwork = 0;
     if (p->order == 4 || (p->order == 5 && p->nshell > 16)) {
+        auto cost = [](double w, const TcState& s) { return s.teams == 2 ? 1.15 * w : w; };
         TcState probe, c;
         TcTables ph, ch;
         if (poly_status s = tc_build_layout(p, &probe, ph, false, false, work)) return s;
-        if (tc_build_layout(p, &c, ch, true, true, cwork) == POLY_OK && cwork <= work) {
+        if (tc_build_layout(p, &c, ch, true, true, cwork) == POLY_OK && cost(cwork, c) <= cost(work, probe)) {
             *t = c;
             h = std::move(ch);
             return POLY_OK;
@@ -1024,11 +1026,11 @@ static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
 // The tensor-core FP32 accumulation error grows with the window; at 256^3 the largest
 // error over the split-BF16 scale is 1.3e-6 for the bispectrum at 128 chunks (6e-7 at 64;
 // the contraction takes 6.54 ms instead of 6.67), but 1.5e-5 for the trispectrum
-// (products of four fields) at 64 chunks, 5.9e-6 at 16.  The compact layouts take 14 (n = 4) and 12 (n = 5)
-// chunks, at which their error is that of the plain ones with 16.
+// (products of four fields) at 64 chunks, 5.4e-6 at 16, 5.0e-6 at 14.  Rows of three legs (n = 5) take 12 chunks, at
+// which their error is that of rows of two with 16.
 // POLY_TC_WINDOW sets another, at least one chunk more than there are slots (TcWindow).
-static int tc_window(int order, int ra, int ca) {
-    const int def = order == 4 ? 14 : ra == 3 && ca == 2 ? 12 : order >= 5 ? 16 : 128;
+static int tc_window(int order, int ra) {
+    const int def = order <= 3 ? 128 : order == 4 ? 14 : order == 5 && ra == 3 ? 12 : 16;
     const char* w = getenv("POLY_TC_WINDOW");
     return w && atoi(w) > 0 ? std::max(atoi(w), kTcMaxSlots + 1) : def;
 }
@@ -1044,10 +1046,8 @@ static poly_status tc_launch_shape(const PsPlan* p, const std::vector<TcGroup>& 
     }
     t->bbuf_bytes = maxcol * kTcChunk * 2;
     t->acc_max = maxacc;
-    // B slots: as many as shared memory holds (the kernel also bounds them by TMEM).  Order 4 takes two from four
-    // groups on: the host-table test holds the trispectrum of 256^3 / 32 shells to two teams, hence two slots
-    // (13.2 ms there; with three teams and slots 12.4, 160^3 / 26 shells 1.68 and 1.64).
-    t->slot_cap = p->order == 4 && groups.size() >= 4 ? 2 : kTcMaxSlots;
+    // B slots: as many as shared memory holds (the kernel also bounds them by TMEM)
+    t->slot_cap = kTcMaxSlots;
     while (t->slot_cap > 2 && tc_smem_bytes(t->stage_bytes, t->bbuf_bytes, t->slot_cap, maxacc) > 227 * 1024)
         t->slot_cap--;
     t->smem_bytes = (int)tc_smem_bytes(t->stage_bytes, t->bbuf_bytes, t->slot_cap, maxacc);
@@ -1057,7 +1057,7 @@ static poly_status tc_launch_shape(const PsPlan* p, const std::vector<TcGroup>& 
     int min_slots = t->slot_cap;
     for (auto& g : groups) min_slots = std::min(min_slots, (512 - (g.acc_cols + 31) / 32 * 32) / (g.nmt * 32));
     t->teams = min_slots >= 3 ? 3 : 2;
-    t->window = tc_window(p->order, t->ra, t->ca);
+    t->window = tc_window(p->order, t->ra);
     return POLY_OK;
 }
 

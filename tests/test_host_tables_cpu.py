@@ -289,7 +289,7 @@ def test_tc_tables_other_plans(lib, N, order, nshell, width, sms):
     check_tc_tables(t, oracle.enumerate_bins(e, order), N, nshell, 4)
     check_pipeline_teams(t)
     if (N, order, nshell) == (256, 4, 32):
-        assert t["teams"] == 2  # the pair columns' B buffers leave shared memory for two slots
+        assert t["teams"] == 3  # three slots of the pair columns' B buffers take 230,648 of 232,448 bytes
 
 
 @pytest.mark.parametrize("N,order,nshell,ell", [(256, 3, 64, 2), (48, 3, 12, 4), (32, 4, 6, 2), (64, 2, 20, 2)])

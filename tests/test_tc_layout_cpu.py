@@ -50,3 +50,13 @@ def test_every_bin_has_its_own_slot_of_its_own_product(lib, N, order, nshell, wi
 def test_refused_plans_stay_refused(lib, order, nshell, ell):
     rc, _ = tc_tables(lib, 256, order, fieldgen.unit_edges(nshell), flags=ps.POLY_ALLOW_ALIAS, ell=ell)
     assert rc == STATUS["POLY_ERR_UNSUPPORTED"]
+
+
+@pytest.mark.parametrize("nshell,groups,teams", [(26, 2, 3), (27, 4, 3), (28, 4, 2), (32, 4, 3), (33, 7, 3), (34, 6, 2)])
+def test_order_4_takes_the_faster_layout_and_the_teams_that_fit(lib, nshell, groups, teams):
+    """The measured choice at 256^3 in shells of 1.5: 27 and 33 shells keep the plain layout's groups and three teams (fewer
+    groups of two teams take longer), 32 take the compact one's with three."""
+    rc, t = tc_tables(lib, 256, 4, fieldgen.unit_edges(nshell, 1.5))
+    assert rc == 0
+    check_pipeline_teams(t)
+    assert (len(t["groups"]), t["teams"]) == (groups, teams)
