@@ -999,21 +999,22 @@ static poly_status tc_build_layout(const PsPlan* p, TcState* t, TcTables& h, boo
     return tc_launch_shape(p, h.groups, t);
 }
 
-// The plain layout, and for orders 4 and 5 the compact one where it is no more work; two producer teams take 1.15 times
-// as long as three (1.05 to 1.14 measured on one layout).  What the plain layout
+// The plain layout; for order 4 the compact one where it is no more work (two producer teams take 1.15 times as long as
+// three: 1.05 to 1.14 measured on one layout), for order 5 the compact one wherever it fits.  What the plain layout
 // refuses stays refused, so the plans taken do not depend on the layout.  Estimates, plain -> compact in ms: n = 4,
 // 256^3 / 32 shells 21.6 -> 13.5, 28 (three teams, two) 16.2 -> 15.7, 34 (the same) 25.8 -> 22.2, but 33 (the same)
 // 21.2 -> 22.3: not taken; 27 the same work, 160^3 / 26 3.5 -> 2.0, 128^3 / 20 0.91 -> 0.86, 64^3 / 10 the same; n = 5,
-// 128^3 / 20 shells 5.1 -> 2.3.  Plans of order 5 up to 16 shells keep the plain layout, which the
-// host-table tests hold them to (not measured there in the compact one).
+// 128^3 / 20 shells 5.1 -> 2.3, 16 1.93 -> 1.18, 12 0.85 -> 0.56, 10 0.56 -> 0.38, 8 0.36 -> 0.29, 5 0.27 -> 0.25,
+// 64^3 / 8 0.094 -> 0.079, 32^3 / 3 the same; its error there is 0.75 times the plain one's.
 static poly_status tc_build_tables(const PsPlan* p, TcState* t, TcTables& h) {
     double work = 0, cwork = 0;
-    if (p->order == 4 || (p->order == 5 && p->nshell > 16)) {
+    if (p->order == 4 || p->order == 5) {
         auto cost = [](double w, const TcState& s) { return s.teams == 2 ? 1.15 * w : w; };
         TcState probe, c;
         TcTables ph, ch;
         if (poly_status s = tc_build_layout(p, &probe, ph, false, false, work)) return s;
-        if (tc_build_layout(p, &c, ch, true, true, cwork) == POLY_OK && cost(cwork, c) <= cost(work, probe)) {
+        if (tc_build_layout(p, &c, ch, true, true, cwork) == POLY_OK &&
+            (p->order == 5 || cost(cwork, c) <= cost(work, probe))) {
             *t = c;
             h = std::move(ch);
             return POLY_OK;

@@ -210,7 +210,7 @@ def factor_wavefronts(t, which):
 def check_tc_tables(t, bins, N, nshell, max_mt, shift=0):
     """shift: the first row factor's slot offset (nshell for a multipole plan's weighted fields)."""
     order = bins.shape[1]
-    ra = 3 if order >= 6 else (2 if order >= 3 else 1)
+    ra = 3 if order >= 5 else (2 if order >= 3 else 1)
     ctas, groups, mtiles, runs, rowf, colf, bm = (t[k] for k in ("ctas", "groups", "mtiles", "runs", "rowf", "colf",
                                                                 "binmap"))
     ng, nchunks = len(groups), (N ** 3 + 31) // 32

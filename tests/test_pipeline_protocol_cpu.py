@@ -191,7 +191,7 @@ def test_short_last_windows_go_wrong(T, S, W, nch):
     assert any(run_drains(T, S, ends, rng, "after") == "stall" for _ in range(2000))
 
 
-@pytest.mark.parametrize("order,nshell,default", [(3, 12, 128), (4, 10, 14), (2, 12, 128)])
+@pytest.mark.parametrize("order,nshell,default", [(3, 12, 128), (4, 10, 14), (2, 12, 128), (5, 8, 12)])
 @pytest.mark.parametrize("env,window", [(None, None), ("1", 5), ("3", 5), ("4", 5), ("5", 5), ("6", 6), ("0", None)])
 def test_window_holds_more_chunks_than_there_are_slots(monkeypatch, order, nshell, default, env, window):
     assert kernel_windows(monkeypatch, order, nshell, 8, env)[0] == (window or default)

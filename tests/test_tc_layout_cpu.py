@@ -1,5 +1,5 @@
 """The tensor-core contraction's compact layout of orders 4 and 5 (rows sorted by their last legs, three-leg rows
-for n = 5 above 16 shells): every bin's slot is the product of exactly its shells, no slot is used twice, and the
+for n = 5): every bin's slot is the product of exactly its shells, no slot is used twice, and the
 plans that the plain layout refuses stay refused.  Host tables only."""
 import numpy as np
 import pytest
@@ -19,7 +19,8 @@ def lib():
 
 @pytest.mark.parametrize("N,order,nshell,width,ell", [
     (256, 4, 32, 1.5, 0), (160, 4, 26, 1.5, 0), (128, 4, 17, 1.0, 0), (48, 4, 3, 1.0, 0), (64, 4, 12, 1.0, 2),
-    (128, 5, 17, 1.0, 0), (128, 5, 20, 1.0, 0), (256, 5, 20, 2.0, 0)])
+    (128, 5, 17, 1.0, 0), (128, 5, 20, 1.0, 0), (256, 5, 20, 2.0, 0), (128, 5, 16, 1.0, 0), (64, 5, 10, 1.0, 0),
+    (48, 5, 3, 1.0, 0), (64, 5, 6, 1.0, 2)])
 def test_every_bin_has_its_own_slot_of_its_own_product(lib, N, order, nshell, width, ell):
     e = fieldgen.unit_edges(nshell, width)
     rc, t = tc_tables(lib, N, order, e, flags=0, ell=ell)
