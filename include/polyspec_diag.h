@@ -161,7 +161,8 @@ int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsig
  * sorted), each listing the bins that produce it.  N, order (2..4), edges,
  * nshell, flags and prec as in poly_plan_create; sms as the device would set it.
  *   sizes[10] (required): entries, entry-bin records, then for the tensor-core
- *   form (order 3, split-BF16; 0 groups when it does not apply): groups, chunks,
+ *   form over columns (m, j) (order 3, split-BF16; 0 groups when it does not
+ *   apply; plans that poly_diag_adj_pairs has tables for run those instead): groups, chunks,
  *   K (shells padded to 32), accumulator columns per buffer, bytes of one B
  *   array, cell ranges per pair of groups, shells without entries, largest
  *   chunk count of a group.  Other pointers may be NULL or host buffers:
@@ -179,6 +180,44 @@ int poly_diag_tc_window(int N, int order, const double* edges, int nshell, unsig
 int poly_diag_adj_tables(int N, int order, const double* edges, int nshell, unsigned flags, int prec, int sms,
                          int64_t* sizes, int32_t* moff, int16_t* ent, int32_t* eoff, int32_t* ebins,
                          int32_t* at_groups, int32_t* at_chunks, int32_t* at_pos);
+
+/*
+ * The host tables of the tensor-core adjoint over pairs of shells (order 3,
+ * split-BF16), computed on the host alone: K = the pairs (i <= j) in chunks of 8
+ * consecutive i by 8 consecutive j, N = the shells m.
+ *   sizes[4] (required): chunks (0: the plan takes the form over columns),
+ *   entries, bytes of the weights, shared memory of a block.  The others may be
+ *   NULL or host buffers:
+ *   chunks int32 [][8]: first j (-1: a chunk without products), first i, first
+ *          column n0, columns nn, byte offset of its weights, first and last
+ *          chunk of its accumulation segment (0 or 1); and in entry s the last
+ *          chunk of segment s.  A segment's first chunk overwrites the sums of
+ *          columns [n0, n0 + nn), the others add to theirs;
+ *   place  int32 [nent][2], entries as in poly_diag_adj_tables: byte offset of the
+ *          weight's first bf16 part and the distance to each of the next two.  Pair (i, j) and
+ *          column m of a chunk lie at (m - n0) / 8 * 1024 + k / 8 * 128 + (m - n0)
+ *          % 8 * 16 + k % 8 * 2 with k = 8 (i - i0) + (j - first j).
+ * Returns a poly_status.
+ */
+int poly_diag_adj_pairs(int N, const double* edges, int nshell, unsigned flags, int64_t* sizes, int32_t* chunks,
+                        int32_t* place);
+
+/*
+ * The host tables of the CUDA-core adjoint (every other plan), computed on the
+ * host alone.  An output block is a run of blk shells m (8 in FP32, 4 in FP64).
+ *   sizes[5] (required): blocks, runs, entries, weights, blk.  The others may be
+ *   NULL or host buffers:
+ *   blocks int32 [][5]: first shell, first run, runs, first record, records;
+ *   segs   int32 [][5]: a, j0, j1, i0, count: `count` records, record r the field
+ *          i0 + r times D_j0 D_a and D_j1 D_a (no D_a for order 3, neither for
+ *          order 2); a block's records follow one another over its runs;
+ *   place  int32 [nent]: where entry e's weight lies: record rec of a block holds
+ *          2 blk weights from (first record + rec) x 2 blk, for j0 and shell
+ *          first + 0 .. blk - 1, then for j1.
+ * Returns a poly_status.
+ */
+int poly_diag_adj_blocks(int N, int order, const double* edges, int nshell, unsigned flags, int prec, int64_t* sizes,
+                         int32_t* blocks, int32_t* segs, int32_t* place);
 
 #ifdef __cplusplus
 }

@@ -414,6 +414,42 @@ static void adj_blocks(int order, int nshell, int blk, const std::vector<int>& m
     std::stable_sort(blocks.begin(), blocks.end(), [](const AdjBlock& x, const AdjBlock& y) { return x.nrec > y.nrec; });
 }
 
+extern "C" int poly_diag_adj_blocks(int N, int order, const double* edges, int nshell, unsigned flags, int prec,
+                                    int64_t* sizes, int32_t* blocks, int32_t* segs, int32_t* place) {
+    if (!sizes) return POLY_ERR_ARG;
+    if (order > 4) return POLY_ERR_UNSUPPORTED;  // as poly_backward
+    try {
+        PsPlan hp;  // host tables only: no device call, no device memory
+        std::vector<short> lines;
+        if (poly_status s = ps_plan_host_tables(&hp, N, 1.0, order, nshell, edges, (poly_precision)prec, flags, 0, lines))
+            return s;
+        std::vector<int> mo, eo, eb, at;
+        std::vector<short4> en;
+        ps_adj_entries(&hp, mo, en, eo, eb);
+        std::vector<AdjBlock> B;
+        std::vector<AdjSeg> G;
+        size_t nweight = 0;
+        const int blk = hp.is_double ? AdjLane<double>::kBlk : AdjLane<float>::kBlk;
+        adj_blocks(order, nshell, blk, mo, en, B, G, at, nweight);
+        const int64_t n[5] = {(int64_t)B.size(), (int64_t)G.size(), (int64_t)at.size(), (int64_t)nweight, blk};
+        for (int i = 0; i < 5; i++) sizes[i] = n[i];
+        for (size_t b = 0; blocks && b < B.size(); b++) {
+            const int32_t v[5] = {B[b].m0, B[b].seg0, B[b].nseg, B[b].rec0, B[b].nrec};
+            std::copy(v, v + 5, blocks + 5 * b);
+        }
+        for (size_t g = 0; segs && g < G.size(); g++) {
+            const int32_t v[5] = {G[g].a, G[g].j0, G[g].j1, G[g].i0, G[g].count};
+            std::copy(v, v + 5, segs + 5 * g);
+        }
+        if (place) std::copy(at.begin(), at.end(), place);
+        return POLY_OK;
+    } catch (const std::bad_alloc&) {
+        return POLY_ERR_ALLOC;
+    } catch (const std::length_error&) {
+        return POLY_ERR_UNSUPPORTED;
+    }
+}
+
 static poly_status adj_prepare(PsPlan* p, AdjTables& A) {
     const int n = p->order;
     std::vector<int> moff, eoff, ebins;

@@ -835,6 +835,13 @@ static void aq_build_tables(const PsPlan* p, const std::vector<int>& ent_m, cons
     S->pairs = true;
 }
 
+// Pairs up to 64 shells (two M tiles' sums and three A slots fill tensor memory), columns (m, j) beyond; and
+// for up to four shells on large grids, where a tile's single chunk leaves the pairs' barriers bare (256^3 / 3
+// shells: gradient 1.16 against 1.10 ms; 5 shells 1.26 against 1.31, 160^3 / 4 shells 0.47 against 0.50).
+static bool aq_takes(int nshell, int64_t ncell) {
+    return nshell <= kAqMaxShells && !(nshell <= 4 && ncell > (int64_t)160 * 160 * 160);
+}
+
 poly_status ps_at_prepare(PsPlan* p, const std::vector<int>& ent_m, const std::vector<short4>& ent, AtState** out) {
     *out = nullptr;
     const int64_t ncell = (int64_t)p->N * p->N * p->N;
@@ -843,10 +850,7 @@ poly_status ps_at_prepare(PsPlan* p, const std::vector<int>& ent_m, const std::v
     if (!S) return POLY_ERR_ALLOC;
     std::vector<int> chunks, pos;
     size_t b_total = 0;
-    // Pairs up to 64 shells (two M tiles' sums and three A slots fill tensor memory), columns (m, j) beyond; and
-    // for up to four shells on large grids, where a tile's single chunk leaves the pairs' barriers bare (256^3 / 3
-    // shells: gradient 1.16 against 1.10 ms; 5 shells 1.26 against 1.31, 160^3 / 4 shells 0.47 against 0.50).
-    if (p->nshell <= kAqMaxShells && !(p->nshell <= 4 && ncell > (int64_t)160 * 160 * 160)) {
+    if (aq_takes(p->nshell, ncell)) {
         aq_build_tables(p, ent_m, ent, S, b_total);
     } else if (poly_status s0 = at_build_tables(p, ent_m, ent, S, chunks, pos, b_total)) {
         delete S;
@@ -943,6 +947,40 @@ extern "C" int poly_diag_adj_tables(int N, int order, const double* edges, int n
     try {
         return diag_adj_tables(N, order, edges, nshell, flags, prec, sms, sizes, moff, ent, eoff, ebins, at_groups,
                                at_chunks, at_pos);
+    } catch (const std::bad_alloc&) {
+        return POLY_ERR_ALLOC;
+    }
+}
+
+extern "C" int poly_diag_adj_pairs(int N, const double* edges, int nshell, unsigned flags, int64_t* sizes, int32_t* chunks,
+                                   int32_t* place) {
+    if (!sizes) return POLY_ERR_ARG;
+    try {
+        PsPlan hp;  // host tables only: no device call, no device memory
+        std::vector<short> lines;
+        if (poly_status s = ps_plan_host_tables(&hp, N, 1.0, 3, nshell, edges, POLY_SPLIT_BF16, flags, 0, lines)) return s;
+        std::vector<int> mo, eo, eb;
+        std::vector<short4> en;
+        ps_adj_entries(&hp, mo, en, eo, eb);
+        std::vector<int> ent_m(en.size());
+        for (int m = 0; m < nshell; m++)
+            for (int e = mo[m]; e < mo[m + 1]; e++) ent_m[e] = m;
+        AtState S;
+        size_t b_total = 0;
+        const bool takes = aq_takes(nshell, (int64_t)N * N * N);
+        if (takes) aq_build_tables(&hp, ent_m, en, &S, b_total);
+        const int64_t n[4] = {(int64_t)S.chunks.size(), (int64_t)S.place.size(), (int64_t)b_total, (int64_t)S.smem};
+        for (int i = 0; i < 4; i++) sizes[i] = takes ? n[i] : 0;
+        for (size_t c = 0; chunks && c < S.chunks.size(); c++) {
+            const AqChunk& C = S.chunks[c];
+            const int32_t v[8] = {C.jb, C.i0, C.n0, C.nn, C.b_off, C.first, C.last, C.end};
+            std::copy(v, v + 8, chunks + 8 * c);
+        }
+        for (size_t e = 0; place && e < S.place.size(); e++) {
+            place[2 * e] = S.place[e].x;
+            place[2 * e + 1] = S.place[e].y;
+        }
+        return POLY_OK;
     } catch (const std::bad_alloc&) {
         return POLY_ERR_ALLOC;
     }

@@ -359,7 +359,7 @@ def check_entries(t, bins, nshell):
 
 
 def check_at_tables(t, nshell):
-    """Tensor-core adjoint: each group's chunks run over its m's in order, one chunk per (m, j block) that
+    """Tensor-core adjoint over columns (m, j): each group's chunks run over its m's in order, one chunk per (m, j block) that
     holds an entry; every entry's weight sits at its own place of its group's B (K-major, 8 x 8 core
     matrices), inside a K block that the group's mask marks."""
     ent, moff, groups, chunks, pos, kp = t["ent"], t["moff"], t["groups"], t["chunks"], t["pos"], t["kp"]
