@@ -341,8 +341,9 @@ poly_status poly_plan_stats(poly_plan plan, poly_stats* out);
  *          poly_plan_counts of a plan with the same N and edges, made earlier.
  *  stream: cudaStream_t; the call is asynchronous on it.
  *
- * Problems whose intermediates do not fit in 32 MiB (roughly nshell * N^3 * 4
- * bytes of fields plus a few MiB) are rejected with POLY_ERR_UNSUPPORTED and a
+ * Problems that count as more than 32 MiB (roughly nshell * N^3 * 4
+ * bytes of fields plus a few MiB for the bins; the count is fixed, and a little
+ * above what the kernels use) are rejected with POLY_ERR_UNSUPPORTED and a
  * message from poly_last_error(); e.g. N = 64 with 16 shells fits, 256^3 does
  * not.  The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current: make it before any stream

@@ -81,8 +81,8 @@ struct Carve {  // 256-byte aligned sub-ranges of the static array
 
 namespace {
 // The limit of this entry point, fixed so that what it takes does not move with the contraction's own
-// layout: its intermediates with the bins cut into tiles of 64 rows (pairs (k1, k2), in the order of their
-// first and last k3) by 64 columns (k3), 4096 sums per tile and split.
+// layout: what its intermediates take with the bins cut into tiles of 64 rows (pairs (k1, k2), in the order of their
+// first and last k3) by 64 columns (k3), 4096 sums per tile and split.  The buffers in use are smaller (checked below).
 struct TileCount {
     size_t tiles = 0, rows = 0, cols = 0, fields = 0;
 };
@@ -172,12 +172,16 @@ static poly_status estimate_noalloc(int N, double L, int nshell, const double* e
                              (size_t)hp.nbins * 8})
             c.take(bytes);
         if (c.used > kNoAllocBytes)
-            return fail(POLY_ERR_UNSUPPORTED, "this problem needs " + std::to_string(c.used >> 20) +
-                                                  " MiB of scratch; the static array holds 32 MiB");
+            return fail(POLY_ERR_UNSUPPORTED, "this problem is over the entry point's size limit: it counts as " +
+                                                  std::to_string(c.used >> 20) + " MiB, of 32 MiB");
     }
+    int dev = 0, sms = 0;
+    if (cudaError_t e = cudaGetDevice(&dev)) return fail(POLY_ERR_CUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
+    if (cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))
+        return fail(POLY_ERR_CUDA, std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e));
     build_cc_tasks(&hp, 0, 0, hp.cc);
     const int64_t one_row = std::max<int64_t>(1, hp.cc.ntask() * cc_span(order, false, 0, order) * 8);
-    const CcLaunch cl = cc_launch_shape(hp.cc, order, nshell, n3 / 32, 152, std::max<int64_t>(1, (int64_t)tile_part / one_row));
+    const CcLaunch cl = cc_launch_shape(hp.cc, order, nshell, n3 / 32, sms, std::max<int64_t>(1, (int64_t)tile_part / one_row));
 
     // layout of the static array
     Carve c;

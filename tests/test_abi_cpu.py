@@ -247,3 +247,11 @@ def test_tensor_checks_run_before_any_library_call():
             call()
     with pytest.raises(ValueError, match="512 elements"):
         plan.estimate_host(np.zeros(500, np.float32))
+
+
+def test_noalloc_refusal_states_the_limit_and_not_a_need(lib):
+    """The size count of poly_estimate_noalloc is a fixed formula: its message must not give it as what the call needs."""
+    edges, counts, x = np.arange(65) + 0.5, np.ones(24432, np.int64), np.zeros(1, np.float32)
+    rc = lib.poly_estimate_noalloc(256, 500.0, 64, edges.ctypes.data, x.ctypes.data, counts.ctypes.data, counts.ctypes.data, None)
+    msg = lib.poly_last_error().decode()
+    assert rc == 6 and "limit" in msg and "of 32 MiB" in msg and "needs" not in msg
