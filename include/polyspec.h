@@ -88,6 +88,14 @@ typedef enum {
  * rounded to its integer map, then summed in 64-bit integers); plans with
  * POLY_ALLOW_ALIAS cannot take that route and return POLY_ERR_COUNT there.
  * It synchronises the device.  On failure *out is set to NULL.
+ *
+ * Range: the shell fields D_s are unnormalised sums over modes, of the order of
+ * N^3 times the field's rms in the shell.  Plans that are not POLY_FP64 form the
+ * products of a bin's n fields at a cell, and sums of them over many cells, in
+ * FP32 (poly_backward: the products of the other n - 1 fields, before the
+ * weights dL/dB / count); results are not finite, or lose bits, where these leave
+ * about 1e-38 .. 3e38.  Strong fields of 256^3 come near it from n = 5 on: scale
+ * delta then, B_b goes with its n-th power.
  */
 poly_status poly_plan_create(poly_plan* out, int N, double L, int order, int nshell, const double* edges,
                              poly_precision prec, unsigned flags);
@@ -110,7 +118,7 @@ poly_status poly_plan_nbins(poly_plan plan, int64_t* nbins);
  * ell even in [0, 8] (POLY_ERR_ARG otherwise; odd multipoles of a real field
  * are not real); ell = 0 is poly_plan_create.  All three precisions; a
  * split-BF16 plan runs the tensor-core contraction with the weighted fields as
- * its rows' first factor (orders 2 to 4, as for monopole plans; 64 unit shells
+ * its rows' first factor (as for monopole plans; 64 unit shells
  * fit, the chunk stages 2 * nshell field rows, and a shell count whose stages
  * leave no shared memory for accumulators is POLY_ERR_UNSUPPORTED).  The plan
  * holds 2 * nshell fields;
