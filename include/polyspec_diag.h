@@ -205,8 +205,9 @@ int poly_diag_adj_pairs(int N, const double* edges, int nshell, unsigned flags, 
 /*
  * The host tables of the CUDA-core adjoint (every other plan), computed on the
  * host alone.  An output block is a run of blk shells m (8 in FP32, 4 in FP64).
- *   sizes[5] (required): blocks, runs, entries, weights, blk.  The others may be
- *   NULL or host buffers:
+ *   sizes[6] (required): blocks, runs, entries, weights, blk, the limit in clock
+ *   cycles of a warp's wait for the units of others.  The others may be NULL or
+ *   host buffers:
  *   blocks int32 [][5]: first shell, first run, runs, first record, records;
  *   segs   int32 [][5]: a, j0, j1, i0, count: `count` records, record r the field
  *          i0 + r times D_j0 D_a and D_j1 D_a (no D_a for order 3, neither for

@@ -112,8 +112,8 @@ struct AdjLane<double> {
 template <typename T, int NPRE>
 __global__ void __launch_bounds__(kAdjThreads, 1)
     adj_blocks_kernel(const T* __restrict__ D, int nshell, int64_t ncell, int ntile, const AdjBlock* __restrict__ blocks,
-                      int nblk, const AdjSeg* __restrict__ segs, const T* __restrict__ w, int nbuf, T* __restrict__ G,
-                      int* __restrict__ err) {
+                      int nblk, const AdjSeg* __restrict__ segs, const T* __restrict__ w, int nbuf, long long wait_cycles,
+                      T* __restrict__ G, int* __restrict__ err) {
     using Ln = AdjLane<T>;
     constexpr int R = Ln::kCells, kBlk = Ln::kBlk, kRec = 2 * kBlk;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -174,11 +174,12 @@ __global__ void __launch_bounds__(kAdjThreads, 1)
         __syncwarp();  // the last unit's weights have been read by every lane
         copy_batch(0);
         copy_batch(1);
-        // tile k's copy has been started, so the barrier's phase before it is over and its parity is unambiguous
+        // the tile before in this buffer is done once other warps' last units of it are, a unit's time at most;
+        // tile k's copy has been started then, so the barrier's phase before it is over and its parity is unambiguous
         const long long t0 = clock64();
         bool ok = true;
         while (ok && !__all_sync(0xffffffffu, s_issued[buf] == k)) {
-            if (*s_abort || clock64() - t0 > tc::kWaitBudgetCycles) *s_abort = 1;
+            if (*s_abort || clock64() - t0 > wait_cycles) *s_abort = 1;
             ok = !__any_sync(0xffffffffu, *s_abort);
         }
         if (!ok || !tc::mbar_wait_warp(&full[buf], (uint32_t)((k / nbuf) & 1), s_abort)) {
@@ -308,6 +309,7 @@ struct AdjTables {
     // the CUDA-core form: output blocks (heaviest first), their runs of records, every entry's weight's place
     void *d_blocks = nullptr, *d_segs = nullptr, *d_place = nullptr;
     int nblk = 0, nbuf = 1;
+    long long wait_cycles = 0;
     size_t nweight = 0, smem = 0;
     int* d_err = nullptr;
     std::vector<int> line_off;  // host copy of the plan's line offsets
@@ -414,6 +416,14 @@ static void adj_blocks(int order, int nshell, int blk, const std::vector<int>& m
     std::stable_sort(blocks.begin(), blocks.end(), [](const AdjBlock& x, const AdjBlock& y) { return x.nrec > y.nrec; });
 }
 
+// Limit of a warp's wait for a tile buffer: the usual budget and four times the longest unit with every warp at work.
+// A record takes 158 issue slots of 16 warps on 4 schedulers in FP32; in FP64 10 instructions of 16 cycles, 16 warps on
+// one unit (1/64 of the FP32 rate).  The largest plans of order 4 (128 shells, 179,000 records) hold a unit for 5e8 cycles.
+static long long adj_wait_cycles(const std::vector<AdjBlock>& blocks, int is_double) {
+    const long long nrec = blocks.empty() ? 0 : blocks[0].nrec;  // heaviest first
+    return tc::kWaitBudgetCycles + 4 * nrec * (is_double ? 10 * 16 * 16 : 158 * 16 / 4);
+}
+
 extern "C" int poly_diag_adj_blocks(int N, int order, const double* edges, int nshell, unsigned flags, int prec,
                                     int64_t* sizes, int32_t* blocks, int32_t* segs, int32_t* place) {
     if (!sizes) return POLY_ERR_ARG;
@@ -431,8 +441,9 @@ extern "C" int poly_diag_adj_blocks(int N, int order, const double* edges, int n
         size_t nweight = 0;
         const int blk = hp.is_double ? AdjLane<double>::kBlk : AdjLane<float>::kBlk;
         adj_blocks(order, nshell, blk, mo, en, B, G, at, nweight);
-        const int64_t n[5] = {(int64_t)B.size(), (int64_t)G.size(), (int64_t)at.size(), (int64_t)nweight, blk};
-        for (int i = 0; i < 5; i++) sizes[i] = n[i];
+        const int64_t n[6] = {(int64_t)B.size(), (int64_t)G.size(), (int64_t)at.size(), (int64_t)nweight, blk,
+                              adj_wait_cycles(B, hp.is_double)};
+        for (int i = 0; i < 6; i++) sizes[i] = n[i];
         for (size_t b = 0; blocks && b < B.size(); b++) {
             const int32_t v[5] = {B[b].m0, B[b].seg0, B[b].nseg, B[b].rec0, B[b].nrec};
             std::copy(v, v + 5, blocks + 5 * b);
@@ -481,6 +492,7 @@ static poly_status adj_prepare(PsPlan* p, AdjTables& A) {
         const int bs = p->is_double ? AdjLane<double>::kBlk : AdjLane<float>::kBlk;
         adj_blocks(n, p->nshell, bs, moff, ent, blocks, segs, place, A.nweight);
         A.nblk = (int)blocks.size();
+        A.wait_cycles = adj_wait_cycles(blocks, p->is_double);
         const size_t tile = (p->is_double ? AdjLane<double>::kChunks : AdjLane<float>::kChunks) * (size_t)p->nshell * 32 * es;
         const size_t rest = (size_t)kAdjWarps * kAdjRing * kAdjBatch * 2 * bs * es + kAdjMaxTiles * 16 + 64;
         A.nbuf = (int)std::max<size_t>(1, std::min<size_t>(kAdjMaxTiles, (224 * 1024 - rest) / tile));
@@ -550,7 +562,7 @@ poly_status ps_backward_impl(PsPlan* p, const void* delta, const double* dL_dB, 
             const int ntile = (int)(ncell / (AdjLane<T>::kChunks * 32));  // N^3 is a multiple of 256
             kern<<<std::min(p->sms, ntile), kAdjThreads, A.smem, st>>>(
                 (const T*)p->d_fields, p->nshell, ncell, ntile, (const AdjBlock*)A.d_blocks, A.nblk, (const AdjSeg*)A.d_segs,
-                (const T*)A.d_w, A.nbuf, (T*)p->d_G, A.d_err);
+                (const T*)A.d_w, A.nbuf, A.wait_cycles, (T*)p->d_G, A.d_err);
             return cudaSuccess;
         };
         if (dbl)

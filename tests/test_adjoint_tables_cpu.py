@@ -98,7 +98,7 @@ def test_other_plans_take_the_columns(lib, N, nshell, width):
 def test_block_tables(lib, N, order, nshell, width, prec):
     fn, P = lib.poly_diag_adj_blocks, ctypes.c_void_p
     fn.argtypes = [ctypes.c_int, ctypes.c_int, P, ctypes.c_int, ctypes.c_uint, ctypes.c_int, P, P, P, P]
-    e, sizes = np.ascontiguousarray(fieldgen.unit_edges(nshell, width), np.float64), np.zeros(5, np.int64)
+    e, sizes = np.ascontiguousarray(fieldgen.unit_edges(nshell, width), np.float64), np.zeros(6, np.int64)
     args = (N, order, e.ctypes.data, nshell, 0, ps.PRECISIONS[prec], sizes.ctypes.data)
     assert fn(*args, None, None, None) == 0
     blocks, segs, place = np.zeros((sizes[0], 5), np.int32), np.zeros((sizes[1], 5), np.int32), np.zeros(sizes[2], np.int32)
@@ -111,6 +111,9 @@ def test_block_tables(lib, N, order, nshell, width, prec):
     weight = np.zeros(nweight)
     weight[place] = w
     G = np.zeros(nshell + blk)
+    # no warp gives up while another works on its unit: its multiply-adds alone, all 16 warps at work, four times
+    unit = int(blocks[:, 4].max()) * 16 * (2 * blk * 16 if prec == "fp64" else 2 * blk * 8 // 4)
+    assert sizes[5] >= 4_000_000_000 + 4 * unit
     assert sorted(blocks[:, 0].tolist()) == list(range(0, nshell, blk)) and np.all(np.diff(blocks[:, 4]) <= 0)  # heavy first
     ranges = sorted((b[3], b[3] + b[4]) for b in blocks.tolist())
     assert all(a[1] <= b[0] and b[0] % 8 == 0 for a, b in zip(ranges, ranges[1:]))  # whole batches of 8 records each
