@@ -582,7 +582,6 @@ poly_status ps_backward_impl(PsPlan* p, const void* delta, const double* dL_dB, 
     const double scale = ps_norm(p) / (double)ncell;
     // forward transforms of all G_m: one batched launch pair when the per-field outputs fit (A.d_Wall), else
     // one field at a time through the plan's workspace
-    const size_t wsz = (size_t)p->N * (2 * p->K + 1) * (p->K + 1);
     const bool batched = A.d_Wall != nullptr;
     if (batched) {
         if ((e = ps_forward_batched(p->N, dbl, p->d_G, p->nshell, p->K, p->d_tw_fwd, A.d_Wall, A.d_fhat_all, nullptr,
@@ -612,7 +611,6 @@ poly_status ps_backward_impl(PsPlan* p, const void* delta, const double* dL_dB, 
         }
         p->launches += 1;
     }
-    (void)wsz;
     // one inverse transform over the union of the shells
     if (!ps_xpre_fits(p, p->nshell, 1)) return POLY_ERR_ARG;
     if ((e = ps_inverse(p->N, dbl, 0, p->d_ghat, p->d_lines, p->d_line_off, p->nshell, 1, p->K, 0, p->N, p->d_tw_inv,

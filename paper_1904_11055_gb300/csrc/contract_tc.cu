@@ -746,7 +746,6 @@ static poly_status tc_build_layout(const PsPlan* p, TcState* t, TcTables& h, boo
     // bank-conflict-free broadcasts).  Single-field rows: 32 consecutive k1.
     // Lanes without a row repeat the block's first row (their accumulator rows are
     // never read).
-    const int ns = p->nshell;
     std::map<int, std::vector<std::pair<RKey, const std::set<CKey>*>>> octets;
     for (auto& kv : rows) {
         const int k1 = kv.first[0];
@@ -774,7 +773,6 @@ static poly_status tc_build_layout(const PsPlan* p, TcState* t, TcTables& h, boo
             blocks.push_back(std::move(blk));
         }
     }
-    (void)ns;
     std::vector<std::pair<std::pair<int, int>, const std::vector<Row>*>> bl;  // (column span, block)
     for (auto& blk : blocks) {
         int lo = 1 << 30, hi = -1;

@@ -36,12 +36,6 @@ PS_DEV void tmem_st8(uint32_t taddr, const uint32_t* v) {
                  "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
 }
-// 32 lanes x 4 columns of 32 bits: this thread's lane, columns taddr.col .. +3
-PS_DEV void tmem_st4(uint32_t taddr, const uint32_t* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
-                 "r"(v[2]), "r"(v[3])
-                 : "memory");
-}
 // 32 lanes x 16 columns of 32 bits: this thread's lane, columns taddr.col .. +15
 PS_DEV void tmem_st16(uint32_t taddr, const uint32_t* v) {
     asm volatile(
@@ -135,17 +129,6 @@ PS_DEV bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Non-blocking test of phase `parity` (acquire when it returns true).
-PS_DEV bool mbar_test(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, "
-        "p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
 // Wait for phase `parity` of `bar`, giving up after the clock budget or when
 // another thread has raised *abort.  Returns false on give-up.
 PS_DEV bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
@@ -189,50 +172,7 @@ PS_DEV void prefetch_tensormap(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)map) : "memory");
 }
 
-// ---- split of an FP32 value into bf16 hi + lo ---------------------------------
-// hi = RN_bf16(v), lo = RN_bf16(v - hi); packs cells (2c, 2c+1) as (low, high) halves.
-PS_DEV void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    float ra = a - __low2float(h), rb = b - __high2float(h);
-    __nv_bfloat162 l = __floats2bfloat162_rn(ra, rb);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-}
-// the same for products x*y, with the residual taken from the exact product (one rounding)
-PS_DEV void split2_prod(float x0, float y0, float x1, float y1, uint32_t& hi, uint32_t& lo) {
-    const float p0 = x0 * y0, p1 = x1 * y1;
-    __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
-    float r0 = fmaf(x0, y0, -__low2float(h)), r1 = fmaf(x1, y1, -__high2float(h));
-    __nv_bfloat162 l = __floats2bfloat162_rn(r0, r1);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-}
-
-// The same for two products at once with packed FP32 pairs (sm_100 family):
-// (x0 y0, x1 y1) -> hi = RN_bf16 pair, lo = RN_bf16 pair of the exact residuals.
-PS_DEV void split2_prod_x2(float x0, float y0, float x1, float y1, uint32_t& hi, uint32_t& lo) {
-    asm("{\n\t"
-        ".reg .b64 xa, ya, pa, na, ra;\n\t"
-        ".reg .f32 p0, p1, r0, r1;\n\t"
-        ".reg .b32 h, n0, n1;\n\t"
-        "mov.b64 xa, {%2, %3};\n\t"
-        "mov.b64 ya, {%4, %5};\n\t"
-        "mul.rn.f32x2 pa, xa, ya;\n\t"
-        "mov.b64 {p0, p1}, pa;\n\t"
-        "cvt.rn.bf16x2.f32 h, p1, p0;\n\t"
-        "xor.b32 n1, h, 0x80008000;\n\t"
-        "shl.b32 n0, n1, 16;\n\t"
-        "and.b32 n1, n1, 0xffff0000;\n\t"
-        "mov.b64 na, {n0, n1};\n\t"
-        "fma.rn.f32x2 ra, xa, ya, na;\n\t"
-        "mov.b64 {r0, r1}, ra;\n\t"
-        "cvt.rn.bf16x2.f32 %1, r1, r0;\n\t"
-        "mov.b32 %0, h;\n\t"
-        "}"
-        : "=r"(hi), "=r"(lo)
-        : "f"(x0), "f"(x1), "f"(y0), "f"(y1));
-}
-
+// ---- split of FP32 values into bf16 hi + lo ---------------------------------
 // Pairs of FP32 values as one 64-bit value (x in the low half): they stay in an aligned register pair, where a
 // packed operation on two separate floats costs moves to build it.
 PS_DEV uint64_t pack2(float x, float y) {
