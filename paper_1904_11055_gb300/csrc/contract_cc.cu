@@ -10,13 +10,15 @@
 // FP32 arithmetic runs in packed pairs, one cell in each half, so that no operand
 // has to be duplicated.
 //
-// What bounds it: FMA issue.  The block over three legs needs 24 shared-memory
+// What bounds it: latency, of the factors' shared-memory loads and of the row and column products in front of the
+// multiply-adds, at the 12 warps an SM that 168 registers a thread leave: at 160^3 / 48 shells 48 % of the issue slots
+// and a third of the FMA pipe are busy.  The shared memory is not the bound: the block over three legs needs 24
 // wavefronts (4 + 4 + 4 fields, conflict-free rows of the cell-tiled layout) for
-// 64 + 16 packed multiply-adds and products, 60 % of the shared memory's rate at
+// 64 + 16 packed multiply-adds and products, 60 % of its rate at
 // the FP32 FMA peak.  (A 64 x 64 tile of products staged in shared memory, 4 x 4
 // per lane and two 16-byte loads per 16 FMAs, is bound by those loads at 50 % of the
 // peak before the products and the idle parts of the tile: 121 ms at 256^3 / 64
-// shells against 36 ms here, 38 TFLOP/s of a measured 56 to 66 TFLOP/s of packed
+// shells against 35.5 ms here, 38 TFLOP/s (31 without the products) of a measured 56 to 66 TFLOP/s of packed
 // FMAs over such register blocks; FP64 at 64^3 / 16 shells 1.05 against 0.45 ms.)
 // The blocks follow the bins closely: 508 tasks x 64 = 1.33 products per bin at
 // 24,432 triangles.

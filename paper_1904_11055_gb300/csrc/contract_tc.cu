@@ -28,7 +28,8 @@
 // slot holds [hi | lo] of cells 0-15, then [hi | lo] of cells 16-31), so the
 // work per chunk is proportional to the number of M tiles.  The rows of a warp
 // come from 8 consecutive k1 and a few consecutive k2, so its shared-memory reads
-// of the factors are bank-conflict-free broadcasts.  The team then writes the
+// of the factors are bank-conflict-free broadcasts (nearly so in the compact layout
+// of orders 4 and 5, tc_build_layout).  The team then writes the
 // column factors (B operand) into shared memory in the K-major core-matrix layout.  Issuer warp m issues the MMAs of M tile m (operands in
 // registers; one elected lane issues and commits).
 #include <cuda.h>
@@ -740,7 +741,8 @@ static poly_status tc_build_layout(const PsPlan* p, TcState* t, TcTables& h, boo
         std::vector<int> cols;    // global column indices, sorted (empty for padding rows)
     };
     // A producer warp takes 32 rows.  Compact layout: the rows sorted by (k2, k3, k1) and cut in 32s; eight lanes
-    // in a row mostly share k2 and k3 and have consecutive k1, conflict-free reads too.  Else pair rows: the rows of one octet of 8
+    // in a row mostly share k2 and k3 and have consecutive k1, so the second and third factors' loads are broadcasts of
+    // 4 wavefronts and the first factor's take 4 to 5.3 (256^3 / 32 shells 5.2).  Else pair rows: the rows of one octet of 8
     // consecutive k1, sorted by (k2, k1) and cut in 32s, so that a warp's rows
     // use at most 8 consecutive k1 and a few consecutive k2 (the factor reads are
     // bank-conflict-free broadcasts).  Single-field rows: 32 consecutive k1.
