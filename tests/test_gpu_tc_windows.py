@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("N,order,nshell", [(64, 3, 16), (64, 4, 10), (48, 3, 12), (64, 2, 12)])
-def test_short_windows(N, order, nshell, monkeypatch):
+def test_short_last_windows(N, order, nshell, monkeypatch):
     e = fieldgen.unit_edges(nshell)
     d = torch.from_numpy(fieldgen.field("lognormal", N, 81, np.float32)).cuda()
     ref, scale = None, None
